@@ -65,11 +65,17 @@ struct hpx_plan_s {
   double* d_cmm;       // [mmax+1] lambda_mm / sin^m(theta) (sign included)
   double* d_coef_c;    // [nalm] recurrence coefficient c_l of mu_l = c_l z mu_{l-1} - mu_{l-2}
   float2* d_coef_cf;   // [nalm] c_l as a double-FP32 pair (hi, lo): the FP32 plans' recurrence
-  double* d_coef_p;    // [nalm] P_l, lambda_l = P_l mu_l
+  double* d_coef_p;    // [nalm] P_l, lambda_l = P_l mu_l (FP64 plans)
+  float2* d_coef_pp;   // [nalm] P_l as a sum of two floats (FP32 plans)
   float* d_coef_pf;    // [nalm] P_l rounded to float
   int* d_lc;           // [mmax+1][npair] first significant l of chain (m, pair)
-  double* d_mu0;       // [mmax+1][npair] mu_{lc-1}
+  double* d_mu0;       // [mmax+1][npair] mu_{lc-1} (FP64 plans)
   double* d_mu1;       // [mmax+1][npair] mu_{lc}
+  float4* d_start;     // [mmax+1][npair] both times 2^104 as double-FP32 pairs (FP32 plans)
+  int* d_lgrid;        // [mmax+1][ngrid] first l from which every chain of a 64-pair group has |mu| >= 2^-kGridExp
+                       // and is past its start (lmax + 1 if some chain never is); FP32 plans
+  int ngrid;           // 64-pair groups
+  float2* d_zf;        // [npair] z as a sum of two floats
   void* d_spec;        // workspace [nbatch][nspec] C2<T>
   void* d_F;           // workspace [nbatch][nring][mmax+1] C2<T>
   void* d_io_map;      // device I/O buffers of the host-buffer entry points (lazy)
@@ -149,9 +155,14 @@ struct hpx_plan_s {
 namespace hpx {
 
 // Significance threshold of the recurrence chains: a chain contributes from
-// the first l at which |mu_l| >= 2^-kSigExp; earlier values are below
-// 2^-kSigExp (about 1.6e-60) and are dropped.
-constexpr int kSigExp = 200;
+// the first l at which |mu_l| >= 2^-e; earlier values are dropped.  FP64 plans
+// keep values down to 2^-200 (about 1.6e-60).  In the others e is where a
+// value's stored or contracted form becomes exactly zero anyway (|mu| grows
+// monotonically up to there), so nothing is lost: below 2^-136 for FP32 and
+// BF16 (df_real flushes 2^9 mu below 2^-126), below 2^-34 for FP16 tables
+// (2^9 |mu| < 2^-25 rounds to zero, the remainder too).  FP16 tables start
+// 6.6% fewer rows that way at Nside 1024, lmax 3071.
+constexpr int kSigExp64 = 200, kSigExp32 = 136, kSigExpHalf = 34;
 
 // Rows (l values) per tensor-core tile of the Legendre analysis; the lambda
 // table's group starts are aligned to this grid relative to m.
@@ -173,23 +184,6 @@ cudaError_t allow_max_smem(F* func) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&maxopt, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, maxopt);
   return e;
-}
-
-// A recurrence value in the contraction's type.  The float case avoids the
-// double-to-float conversion instruction, which on this GPU issues to the same
-// scarce FP64 pipe as the recurrence: sign, exponent and top 24 significand
-// bits are moved with integer operations (rounded half up in magnitude), and
-// |x| < 2^-126 becomes 0.  |x| here is far below 2^128.  Every lambda table
-// and kernel converts with this one function, so their values agree bit for
-// bit.
-template <typename T> __device__ __forceinline__ T to_real(double x);
-template <> __device__ __forceinline__ double to_real<double>(double x) { return x; }
-template <> __device__ __forceinline__ float to_real<float>(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned ahi = hi & 0x7fffffffu;
-  unsigned f = __funnelshift_l(lo, ahi, 3) + 0x40000000u + ((lo >> 28) & 1u);
-  f = (ahi < (897u << 20)) ? 0u : (f | (hi & 0x80000000u));
-  return __uint_as_float(f);
 }
 
 // Double-FP32 numbers (Dekker's double-length arithmetic, 1971): a value is
@@ -227,27 +221,44 @@ __device__ __forceinline__ Df df_step(Df t, Df n1, Df n2) {
   const float h = __fadd_rn(s, f);
   return Df{h, __fsub_rn(f, __fsub_rn(h, s))};
 }
-// the float value of a scaled pair: hi 2^-104, and 0 below 2^-126 (as to_real)
+// the float value of a scaled pair: hi 2^-104, and 0 below 2^-126
 __device__ __forceinline__ float df_real(Df x) { return fabsf(x.hi) < 0x1p-22f ? 0.f : __fmul_rn(x.hi, 0x1p-104f); }
 
-// One recurrence chain mu_l = c_l z mu_{l-1} - mu_{l-2} of a plan with real
-// type T, restarted at its first significant l (lc) with the stored
-// (mu_{lc-1}, mu_lc) and zero before: FP64 for FP64 plans, double-FP32 for
-// the others (whose results need FP32 accuracy; the pair's ~2^-46 error per
-// step stays far below it over any chain).  C is the coefficient type the
-// kernels stage (8 bytes either way).  step() returns mu_l as a T; every
-// kernel and table of a plan steps with it, so their values agree bit for
-// bit.
-template <typename T> struct Recur;
-template <> struct Recur<double> {
-  using C = double;
+// One recurrence chain mu_l = c_l z mu_{l-1} - mu_{l-2}, restarted at its first
+// significant l (lc) with the stored (mu_{lc-1}, mu_lc) and zero before.  FP64
+// plans (RecurD) step in FP64.  The others step in two phases:
+//
+// * General (RecurG): double-FP32, 19 FP32 operations a step, 3 more for the
+//   value; good for any magnitude, so it carries a chain through its growth.
+// * Grid (GridState), from the group's grid start on: the value is s + f with
+//   s a multiple of a fixed quantum u (2^-18 in mu).  The product is split
+//   into its multiple of u, q = (p s1 + C) - C with C = 1.5 2^23 u, and the
+//   exact rest (one FMA), so s = q - s2 is exact and needs no TwoSum; f takes
+//   the rest and the first-order terms in plain FP32.  |mu| is at most 15.4
+//   for Nside <= 2048 (m = 0 on the first rings), so |s| < 2^23 u and q, of at
+//   most twice that, stays a multiple of u / 2.  s absorbs f's whole quanta
+//   every 16 steps (regrid), so f stays within tens of u and a step adds about
+//   2^-39 absolute error.  11 operations a step and one for the value.
+//
+// A chain changes phase at the grid start of its 64-pair group: every chain of
+// the group has started and has |mu| >= 2^-4 (it grows from there, and a step's
+// error with it), aligned up to the 32-step blocks m + 32 k.  The groups of
+// the first Npair / 32 pairs never do from Nside 512 on: so near the pole a
+// step's error grows linearly in l.  Simulated against extended precision
+// (relative L2 over l of the worst chain): 2^-24 at Nside 2048 / lmax 6143,
+// 2^-24 .. 2^-31 elsewhere, median 2^-34, where rounding the values to FP32
+// gives 2^-26.  92% of
+// the steps at Nside 2048 / lmax 6143 are grid steps, 78% at Nside 512 / lmax
+// 1024.  Every FP32 kernel and table takes the same steps (operations rounded
+// one by one, scalar or two chains packed), so their values agree bit for bit.
+struct RecurD {
   double z = 0.0, s0 = 0.0, s1 = 0.0, n1 = 0.0, n2 = 0.0;
   __device__ __forceinline__ void start(double z_, double s0_, double s1_) {
     z = z_;
     s0 = s0_;
     s1 = s1_;
   }
-  __device__ __forceinline__ double step(C c, int l, int lc) {
+  __device__ __forceinline__ double step(double c, int l, int lc) {
     double mu = fma(c * z, n1, -n2);
     if (l == lc) {
       mu = s1;
@@ -258,33 +269,325 @@ template <> struct Recur<double> {
     return mu;
   }
 };
-template <> struct Recur<float> {
-  using C = float2;
-  Df z{0.f, 0.f}, s0{0.f, 0.f}, s1{0.f, 0.f}, n1{0.f, 0.f}, n2{0.f, 0.f};
-  __device__ __forceinline__ void start(double z_, double s0_, double s1_) {
-    z = df_of(z_);
-    s0 = df_of(s0_ * kDfUp);
-    s1 = df_of(s1_ * kDfUp);
-  }
-  __device__ __forceinline__ float step(C c, int l, int lc) {
-    Df mu = df_step(df_mul(Df{c.x, c.y}, z), n1, n2);
-    if (l == lc) {
-      mu = s1;
-      n1 = s0;
-    }
+
+constexpr int kGridExp = 4;     // see above
+constexpr int kGridBlock = 32;  // the grid start's alignment relative to m
+constexpr int kRegrid = 16;     // steps between regrids
+constexpr float kGridC = 48.f;  // 1.5 2^23 u for u = 2^-18 (times the scale of scaled chains)
+// groups of 64 pairs (p0: the first) that stay in the general phase
+__host__ __device__ inline bool grid_never(int p0, int npair) { return npair >= 1024 && p0 < npair / 32; }
+// the aligned grid start of a group whose recorded one is lg
+__host__ __device__ inline int grid_start(int m, int lg) {
+  return m + (lg - m + kGridBlock - 1) / kGridBlock * kGridBlock;
+}
+
+struct GridState {
+  float s1, f1, s2, f2;
+};
+__device__ __forceinline__ void grid_split(Df x, float C, float& s, float& f) {
+  const float h = __fmul_rn(x.hi, 0x1p-104f);  // exact: |mu| >= 2^-4 here, and n2 has grown alongside
+  s = __fsub_rn(__fadd_rn(h, C), C);
+  f = __fadd_rn(__fsub_rn(h, s), __fmul_rn(x.lo, 0x1p-104f));
+}
+__device__ __forceinline__ GridState grid_enter(Df n1, Df n2, float C) {
+  GridState g;
+  grid_split(n1, C, g.s1, g.f1);
+  grid_split(n2, C, g.s2, g.f2);
+  return g;
+}
+__device__ __forceinline__ void regrid(GridState& g, float C) {
+  const float k1 = __fsub_rn(__fadd_rn(g.f1, C), C), k2 = __fsub_rn(__fadd_rn(g.f2, C), C);
+  g.s1 = __fadd_rn(g.s1, k1);
+  g.f1 = __fsub_rn(g.f1, k1);
+  g.s2 = __fadd_rn(g.s2, k2);
+  g.f2 = __fsub_rn(g.f2, k2);
+}
+__device__ __forceinline__ float grid_step(GridState& g, Df t, float C) {  // t = c_l z
+  const float q = __fsub_rn(__fmaf_rn(t.hi, g.s1, C), C);
+  float r = __fmaf_rn(t.hi, g.s1, -q);
+  const float s = __fsub_rn(q, g.s2);
+  r = __fmaf_rn(t.hi, g.f1, r);
+  r = __fmaf_rn(t.lo, g.s1, r);
+  const float f = __fsub_rn(r, g.f2);
+  g.s2 = g.s1;
+  g.f2 = g.f1;
+  g.s1 = s;
+  g.f1 = f;
+  return __fadd_rn(s, f);
+}
+
+// Two chains a thread, packed: each operation is one instruction for both
+// (f32x2), rounded as the scalar one.
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 pk2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpk2(F2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ F2 neg2(F2 v) {
+  float a, b;
+  unpk2(v, a, b);
+  return pk2(-a, -b);
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+struct GridState2 {
+  F2 s1 = 0, f1 = 0, s2 = 0, f2 = 0;
+};
+__device__ __forceinline__ GridState2 grid_pack(const GridState& a, const GridState& b) {
+  return GridState2{pk2(a.s1, b.s1), pk2(a.f1, b.f1), pk2(a.s2, b.s2), pk2(a.f2, b.f2)};
+}
+__device__ __forceinline__ void grid_unpack(const GridState2& g, GridState& a, GridState& b) {
+  unpk2(g.s1, a.s1, b.s1);
+  unpk2(g.f1, a.f1, b.f1);
+  unpk2(g.s2, a.s2, b.s2);
+  unpk2(g.f2, a.f2, b.f2);
+}
+__device__ __forceinline__ void regrid(GridState2& g, F2 C) {
+  const F2 nC = neg2(C), k1 = add2(add2(g.f1, C), nC), k2 = add2(add2(g.f2, C), nC);
+  g.s1 = add2(g.s1, k1);
+  g.f1 = add2(g.f1, neg2(k1));
+  g.s2 = add2(g.s2, k2);
+  g.f2 = add2(g.f2, neg2(k2));
+}
+// c4: the step's coefficient pair, each part twice (hi, hi, lo, lo)
+__device__ __forceinline__ F2 grid_step(GridState2& g, float4 c4, F2 zh, F2 zl, F2 C) {
+  const F2 ch = pk2(c4.x, c4.y), cl = pk2(c4.z, c4.w);
+  const F2 p = mul2(ch, zh);
+  F2 e = fma2(ch, zh, neg2(p));
+  e = fma2(ch, zl, e);
+  e = fma2(cl, zh, e);
+  const F2 q = add2(fma2(p, g.s1, C), neg2(C));
+  F2 r = fma2(p, g.s1, neg2(q));
+  const F2 s = add2(q, neg2(g.s2));
+  r = fma2(p, g.f1, r);
+  r = fma2(e, g.s1, r);
+  const F2 f = add2(r, neg2(g.f2));
+  g.s2 = g.s1;
+  g.f2 = g.f1;
+  g.s1 = s;
+  g.f1 = f;
+  return add2(s, f);
+}
+
+// the general phase of one chain
+struct RecurG {
+  Df n1{0.f, 0.f}, n2{0.f, 0.f};
+  __device__ __forceinline__ float step(float2 c, Df z) { return step(df_mul(Df{c.x, c.y}, z)); }
+  __device__ __forceinline__ float step(Df t) {  // t = c_l z
+    const Df mu = df_step(t, n1, n2);
     n2 = n1;
     n1 = mu;
     return df_real(mu);
   }
+  // the step l == lc, from the stored (mu_{lc-1}, mu_lc) 2^104 as (hi, lo, hi, lo)
+  __device__ __forceinline__ float start(float4 st) {
+    n2 = Df{st.x, st.y};
+    n1 = Df{st.z, st.w};
+    return df_real(n1);
+  }
 };
-template <typename T> using RecCoef = typename Recur<T>::C;
-// the plan's coefficients in the form Recur<T> stages
-template <typename T> inline const RecCoef<T>* rec_coefs(const hpx_plan_s* p) {
-  return reinterpret_cast<const RecCoef<T>*>(sizeof(T) == 4 ? (const void*)p->d_coef_cf : (const void*)p->d_coef_c);
-}
+
+// One chain through both phases, step by step from some l = m + 32 k at or
+// before its start (table fills): the scalar form of what the kernels do.
+struct Chain {
+  RecurG rc;
+  GridState g{0.f, 0.f, 0.f, 0.f};
+  float4 st{0.f, 0.f, 0.f, 0.f};
+  Df z{0.f, 0.f};
+  float C = kGridC;
+  int m = 0, lc = 0x7fffffff, lg = 0x7fffffff;  // lg: aligned grid start of the chain's group
+  const float2* c = nullptr;
+  __device__ __forceinline__ float step(int l) {
+    if (l < lg) return l == lc ? rc.start(st) : rc.step(c[l], z);
+    if (l == lg) g = grid_enter(rc.n1, rc.n2, C);
+    else if (((l - m) & (kRegrid - 1)) == 0) regrid(g, C);
+    return grid_step(g, df_mul(Df{c[l].x, c[l].y}, z), C);
+  }
+};
 
 __host__ __device__ inline long long alm_base(int lmax, int m) {  // index(l = 0, m); index(l, m) = alm_base + l
   return (long long)m * (2 * lmax + 1 - m) / 2;
+}
+
+// the chain (m, p) with values scaled by S (a power of two); zeros for p >= npair
+template <int S>
+__device__ __forceinline__ Chain chain_at(const RingInfo* __restrict__ rings, const float2* __restrict__ coef_cf,
+                                          const int* __restrict__ lc_tab, const float4* __restrict__ start,
+                                          const int* __restrict__ lgrid, int ngrid, int lmax, int npair, int m, int p) {
+  Chain ch;
+  ch.m = m;
+  ch.c = coef_cf + alm_base(lmax, m);
+  ch.C = kGridC * S;
+  if (p < npair) {
+    const long long ci = (long long)m * npair + p;
+    ch.lc = lc_tab[ci];
+    ch.lg = grid_start(m, lgrid[(long long)m * ngrid + (p >> 6)]);
+    ch.z = df_of(rings[p].z);
+    const float4 v = start[ci];
+    ch.st = make_float4(S * v.x, S * v.y, S * v.z, S * v.w);
+  }
+  return ch;
+}
+
+// G_m(y) = w_y exp(-i m phi_{0,y}) X_y[m mod N_y], with X_y[N - k] = conj X_y[k]
+// (the m-aliasing fold of Eq. 26 for m >= N_y / 2).
+template <typename T>
+__device__ __forceinline__ C2<T> ring_coef(const C2<T>* __restrict__ spec, const C2<T>* __restrict__ etab,
+                                           const RingInfo& R, int m, int b, long long nspec, int use_w) {
+  const int N = R.nphi, H = N >> 1;
+  const int k = m % N;
+  const C2<T>* X = spec + (long long)b * nspec + R.specoff;
+  const C2<T> x = (k <= H) ? X[k] : cconj(X[N - k]);
+  C2<T> g = cmul(x, etab[R.etab + ((long long)R.sigma * m) % (2LL * N)]);
+  if (use_w) g = cscale(g, (T)R.w);
+  return g;
+}
+
+// A general step of a chain in the state registers of both phases (n1, n2 as
+// hi and lo parts).  A chain that has not started (l < lc) holds its start
+// values there and gives zero; at lc it gives the second of them.  WAIT false:
+// the chain is past its start.
+template <bool WAIT>
+__device__ __forceinline__ float general_step(GridState& g, Df t, int l, int lc) {  // t = c_l z
+  RecurG r{Df{g.s1, g.f1}, Df{g.s2, g.f2}};
+  float v = r.step(t);
+  if constexpr (WAIT) {
+    const bool run = l > lc;
+    if (run) g = GridState{r.n1.hi, r.n1.lo, r.n2.hi, r.n2.lo};
+    v = run ? v : l == lc ? df_real(Df{g.s1, g.f1}) : 0.f;
+  } else {
+    g = GridState{r.n1.hi, r.n1.lo, r.n2.hi, r.n2.lo};
+  }
+  return v;
+}
+// the state before the start, from the stored (mu_{lc-1}, mu_lc) as (hi, lo, hi, lo)
+__device__ __forceinline__ GridState start_state(float4 st, float scale) {
+  return GridState{scale * st.z, scale * st.w, scale * st.x, scale * st.y};
+}
+
+// The two chains of one lane.  One state serves both phases: general before
+// the group's grid start, grid (s, f) from it on.  Grid steps take both chains
+// packed (f32x2).  Values are scaled by S, a power of two.
+template <int S>
+struct Chains2 {
+  static constexpr float kC = kGridC * S;
+  GridState2 g;
+  F2 zh, zl;
+  int lca = 0x7fffffff, lcb = 0x7fffffff;  // starts (INT_MAX: none)
+  int lmin, lmax_c;  // the warp's earliest and latest start
+  int lg = 0x7fffffff;  // the group's aligned grid start
+  int m;
+
+  __device__ __forceinline__ void init(const float2* __restrict__ zf, const int* __restrict__ lc_tab,
+                                       const float4* __restrict__ start, const int* __restrict__ lgrid, int ngrid,
+                                       int npair, int lmax, int m_, int grp, int lane) {
+    m = m_;
+    const int pa = grp * 64 + lane, pb = pa + 32;
+    const long long ca = (long long)m * npair + pa;
+    float2 za = make_float2(0.f, 0.f), zb = za;
+    GridState a{0.f, 0.f, 0.f, 0.f}, b = a;
+    if (pa < npair) {
+      lca = lc_tab[ca];
+      za = zf[pa];
+      a = start_state(start[ca], (float)S);
+      lg = grid_start(m, lgrid[(long long)m * ngrid + grp]);
+    }
+    if (pb < npair) {
+      lcb = lc_tab[ca + 32];
+      zb = zf[pb];
+      b = start_state(start[ca + 32], (float)S);
+    }
+    if (lca > lmax) lca = 0x7fffffff;
+    if (lcb > lmax) lcb = 0x7fffffff;
+    zh = pk2(za.x, zb.x);
+    zl = pk2(za.y, zb.y);
+    g = grid_pack(a, b);
+    lmin = __reduce_min_sync(0xffffffffu, min(lca, lcb));
+    lmax_c = __reduce_max_sync(0xffffffffu, max(lca, lcb));
+    lg = __reduce_min_sync(0xffffffffu, lg);  // lanes past npair follow the group
+  }
+
+  // mu_l .. mu_{l+7} of both chains, l - m a multiple of 8; cz: c_l .. c_{l+7}
+  // as (hi, hi, lo, lo)
+  __device__ __forceinline__ void steps8(const float4* cz, int l, float (&va)[8], float (&vb)[8]) {
+    const F2 C = pk2(kC, kC);
+    if (l > lg) {
+      if (((l - m) & (kRegrid - 1)) == 0) regrid(g, C);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) unpk2(grid_step(g, cz[u], zh, zl, C), va[u], vb[u]);
+      return;
+    }
+    GridState a, b;
+    grid_unpack(g, a, b);
+    if (l == lg) {
+      g = grid_pack(grid_enter(Df{a.s1, a.f1}, Df{a.s2, a.f2}, kC), grid_enter(Df{b.s1, b.f1}, Df{b.s2, b.f2}, kC));
+#pragma unroll
+      for (int u = 0; u < 8; ++u) unpk2(grid_step(g, cz[u], zh, zl, C), va[u], vb[u]);
+      return;
+    }
+    Df za, zb;
+    unpk2(zh, za.hi, zb.hi);
+    unpk2(zl, za.lo, zb.lo);
+    // the products c z first: they do not wait on the chains
+    Df ta[8], tb[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const Df c{cz[u].x, cz[u].z};
+      ta[u] = df_mul(c, za);
+      tb[u] = df_mul(c, zb);
+    }
+    if (lmax_c >= l) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        va[u] = general_step<true>(a, ta[u], l + u, lca);
+        vb[u] = general_step<true>(b, tb[u], l + u, lcb);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        va[u] = general_step<false>(a, ta[u], l + u, lca);
+        vb[u] = general_step<false>(b, tb[u], l + u, lcb);
+      }
+    }
+    g = grid_pack(a, b);
+  }
+};
+
+// The plan-resident lambda table (HPX_PLAN_LAMBDA_TABLE): for every m and
+// every group g of 32 consecutive ring pairs, rows l = lstart(m,g)..lmax of 32
+// values mu_l (one per pair of the group), lstart = the group's earliest chain
+// start; row r of (m, g) at tab[off(m,g) + 32 r].  Written once at plan time
+// by the same FP64 recurrence and conversion as the recomputing kernels.
+template <typename T> struct LamTab {
+  const T* tab;
+  const long long* off;
+  const int* lstart;
+  int ngroup;
+};
+
+template <typename T>
+inline LamTab<T> lam_tab(const hpx_plan_s* p) {
+  LamTab<T> tb;
+  tb.tab = static_cast<const T*>(p->d_tab);
+  tb.off = p->d_tab_off;
+  tb.lstart = p->d_tab_lstart;
+  tb.ngroup = p->ngroup;
+  return tb;
 }
 
 // launchers (defined in hpx_fft.cu / hpx_legendre.cu)
@@ -299,6 +602,11 @@ cudaError_t launch_analysis(const hpx_plan_s* p, T* alm, bool use_weight, double
                             int* nlaunch);
 template <typename T>
 cudaError_t launch_synthesis(const hpx_plan_s* p, const T* alm, double mfac, cudaStream_t s, int* nlaunch);
+// FP64: hpx_legendre.cu; FP32: hpx_legendre_f32.cu
+template <> cudaError_t launch_analysis<double>(const hpx_plan_s*, double*, bool, double, cudaStream_t, int*);
+template <> cudaError_t launch_analysis<float>(const hpx_plan_s*, float*, bool, double, cudaStream_t, int*);
+template <> cudaError_t launch_synthesis<double>(const hpx_plan_s*, const double*, double, cudaStream_t, int*);
+template <> cudaError_t launch_synthesis<float>(const hpx_plan_s*, const float*, double, cudaStream_t, int*);
 
 // plan-time table builders (hpx_fft.cu, hpx_legendre.cu)
 template <typename T>

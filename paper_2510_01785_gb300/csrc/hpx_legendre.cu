@@ -13,10 +13,11 @@
 //
 // Exponent rescaling: a plan-time pass runs every (m, ring) chain in a
 // (mantissa, 2^(-512 k)) representation from lambda_mm until it first
-// reaches 2^-200 and records l_c and (mu_{l_c-1}, mu_{l_c}).  Values before
-// l_c are below 2^-193 and are dropped; after l_c they stay within the
-// double range, so the per-transform kernels run the plain recurrence from
-// the recorded state and skip the dropped part of every chain.
+// reaches 2^-200 (FP32 plans: the larger thresholds below which their values
+// are zero anyway, see kSigExp64) and records l_c and (mu_{l_c-1}, mu_{l_c}).
+// Values before l_c are dropped; after l_c they stay within the double range,
+// so the per-transform kernels run the plain recurrence from the recorded
+// state and skip the dropped part of every chain.
 //
 // Contraction with the rings (analysis) or coefficients (synthesis) uses the
 // north/south symmetry lambda_lm(-z) = (-1)^(l+m) lambda_lm(z): each chain
@@ -32,6 +33,8 @@
 namespace cg = cooperative_groups;
 
 namespace hpx {
+
+using T = double;  // the transform kernels of this file serve FP64 plans; hpx_legendre_f32.cu has the FP32 ones
 
 constexpr int LB = 32;  // l values per block of the recurrence
 
@@ -61,14 +64,20 @@ __global__ void k_lambda_mm_prefactor(int mmax, double* cmm) {
 }
 
 // c_l and P_l of the rescaled recurrence for every (l, m); packed like alm.
-__global__ void k_recurrence_coefs(int lmax, int mmax, double* coef_c, double* coef_p,
+// coef_p (FP64 plans) or coef_pp (the others: hi + lo).
+__global__ void k_recurrence_coefs(int lmax, int mmax, double* coef_c, double* coef_p, float2* coef_pp,
                                    float* coef_pf) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m > mmax) return;
   const long long base = (long long)m * (2 * lmax + 1 - m) / 2;
+  auto put = [&](int l, double P) {
+    const float hi = (float)P;
+    if (coef_p) coef_p[base + l] = P;
+    if (coef_pp) coef_pp[base + l] = make_float2(hi, (float)(P - (double)hi));
+    coef_pf[base + l] = hi;
+  };
   coef_c[base + m] = 0.0;
-  coef_p[base + m] = 1.0;
-  coef_pf[base + m] = 1.0f;
+  put(m, 1.0);
   double p1 = 1.0, p2 = 1.0, a_prev = 0.0;  // P_{l-1}, P_{l-2}, alpha_{l-1}
   const double md = m;
   for (int l = m + 1; l <= lmax; ++l) {
@@ -83,19 +92,23 @@ __global__ void k_recurrence_coefs(int lmax, int mmax, double* coef_c, double* c
       c = a * p1 / P;
     }
     coef_c[base + l] = c;
-    coef_p[base + l] = P;
-    coef_pf[base + l] = (float)P;
+    put(l, P);
     p2 = p1;
     p1 = P;
     a_prev = a;
   }
 }
 
-// Start of every chain (m, pair): the first l at which |mu_l| >= 2^-200,
+// Start of every chain (m, pair): the first l at which |mu_l| >= 2^-sig,
 // with (mu_{l-1}, mu_l) there; l_c = lmax + 1 if the chain never gets there.
+// FP32 plans (lgrid given, zeroed before): also, per group of 64 pairs, the
+// largest over its chains of the first l past l_c at which |mu_l| >=
+// 2^-kGridExp (lmax + 1 where a chain never gets there; a plain FP32
+// recurrence finds it).
 __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* __restrict__ cmm,
-                             const double* __restrict__ coef_c, int lmax, int npair, int* lc_tab,
-                             double* mu0_tab, double* mu1_tab) {
+                             const double* __restrict__ coef_c, const float2* __restrict__ coef_cf, int lmax,
+                             int npair, int sig, int* lc_tab, double* mu0_tab, double* mu1_tab,
+                             float4* __restrict__ start, int* __restrict__ lgrid, int ngrid) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (p >= npair) return;
@@ -120,7 +133,8 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
   const double v0 = frexp(cmm[m] * rm, &e1);
   const long long E = er + (long long)m * es + e1;  // |lambda_mm| in [2^(E-1), 2^E)
   long long k = 0;
-  if (E < -(kSigExp - 1)) k = (-(kSigExp - 1) - E + 511) / 512;
+  if (E < -(sig - 1)) k = (-(sig - 1) - E + 511) / 512;
+  const double up = ldexp(1.0, 512 - sig);
   double mu1 = ldexp(v0, (int)(E + 512 * k)), mu2 = 0.0;
   int l = m;
   const long long base = (long long)m * (2 * lmax + 1 - m) / 2;
@@ -129,41 +143,46 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
     const double mu = fma(coef_c[base + l] * z, mu1, -mu2);
     mu2 = mu1;
     mu1 = mu;
-    if (fabs(mu1) >= 0x1p312) {
+    if (fabs(mu1) >= up) {
       mu1 *= 0x1p-512;
       mu2 *= 0x1p-512;
       --k;
     }
   }
   const long long ci = (long long)m * npair + p;
-  if (k > 0) {
-    lc_tab[ci] = lmax + 1;
-    mu0_tab[ci] = 0.0;
-    mu1_tab[ci] = 0.0;
-  } else {
-    lc_tab[ci] = l;
+  if (k > 0) mu1 = mu2 = 0.0;
+  lc_tab[ci] = k > 0 ? lmax + 1 : l;
+  if (!start) {
     mu0_tab[ci] = mu2;
     mu1_tab[ci] = mu1;
+    return;
   }
+  const Df d0 = df_of(mu2 * kDfUp), d1 = df_of(mu1 * kDfUp);
+  start[ci] = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
+  int lg = lmax + 1;
+  if (k <= 0 && !grid_never(p & ~63, npair)) {
+    const float zf = (float)z;
+    float x1 = (float)(mu1 * 0x1p100), x2 = (float)(mu2 * 0x1p100);
+    lg = l;
+    while (lg <= lmax && fabsf(x1) < 0x1p100f * (1.f / (1 << kGridExp))) {
+      ++lg;
+      if (lg > lmax) break;
+      const float x = fmaf(coef_cf[base + lg].x * zf, x1, -x2);
+      x2 = x1;
+      x1 = x;
+    }
+    lg = max(lg, l + 1);
+  }
+  // one atomic per half group: the lanes of a warp with pairs share a 64-pair group
+  const int left = npair - (p & ~31);
+  const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+  lg = __reduce_max_sync(mask, lg);
+  if ((threadIdx.x & 31) == 0) atomicMax(lgrid + (long long)m * ngrid + (p >> 6), lg);
 }
 
 // ---------------------------------------------------------------------------
 // analysis
 // ---------------------------------------------------------------------------
-// G_m(y) = w_y exp(-i m phi_{0,y}) X_y[m mod N_y], with X_y[N - k] = conj X_y[k]
-// (the m-aliasing fold of Eq. 26 for m >= N_y / 2).
-template <typename T>
-__device__ __forceinline__ C2<T> ring_coef(const C2<T>* __restrict__ spec, const C2<T>* __restrict__ etab,
-                                           const RingInfo& R, int m, int b, long long nspec, int use_w) {
-  const int N = R.nphi, H = N >> 1;
-  const int k = m % N;
-  const C2<T>* X = spec + (long long)b * nspec + R.specoff;
-  const C2<T> x = (k <= H) ? X[k] : cconj(X[N - k]);
-  C2<T> g = cmul(x, etab[R.etab + ((long long)R.sigma * m) % (2LL * N)]);
-  if (use_w) g = cscale(g, (T)R.w);
-  return g;
-}
-
 // Lane tiling of the (LB x 2CP) output block of one warp: each lane owns LPL
 // consecutive l and CPL consecutive real components.
 template <int C2N> struct LaneTile;
@@ -173,29 +192,17 @@ template <> struct LaneTile<8> { static constexpr int CPL = 4, LPL = 2; };
 template <> struct LaneTile<16> { static constexpr int CPL = 4, LPL = 4; };
 template <> struct LaneTile<32> { static constexpr int CPL = 8, LPL = 4; };
 
-template <typename T> struct MuStride { static constexpr int v = LB + 16 / (int)sizeof(T); };
+constexpr int kMuStride = LB + 16 / (int)sizeof(T);
 
 // S/A coefficients, mu rows (each warp's partial sums of a block reuse its own
 // 32 rows once it has read them), the double-buffered block partials, c_l
-template <typename T, int CP>
+template <int CP>
 size_t analysis_smem(int nthr) {
   constexpr int C2N = 2 * CP;
-  static_assert(LB * C2N <= 32 * MuStride<T>::v, "partials fit a warp's mu rows");
-  return sizeof(T) * ((size_t)nthr * 2 * C2N + (size_t)nthr * MuStride<T>::v + 2 * LB * C2N) +
+  static_assert(LB * C2N <= 32 * kMuStride, "partials fit a warp's mu rows");
+  return sizeof(T) * ((size_t)nthr * 2 * C2N + (size_t)nthr * kMuStride + 2 * LB * C2N) +
          sizeof(double) * 2 * LB;
 }
-
-// The plan-resident lambda table (HPX_PLAN_LAMBDA_TABLE): for every m and
-// every group g of 32 consecutive ring pairs, rows l = lstart(m,g)..lmax of 32
-// values mu_l (one per pair of the group), lstart = the group's earliest chain
-// start; row r of (m, g) at tab[off(m,g) + 32 r].  Written once at plan time
-// by the same FP64 recurrence and conversion as the recomputing kernels.
-template <typename T> struct LamTab {
-  const T* tab;
-  const long long* off;
-  const int* lstart;
-  int ngroup;
-};
 
 // One cluster per m, one recurrence chain per thread.  Warps take 32
 // consecutive ring pairs (similar start l, so few idle lanes) and are dealt
@@ -207,10 +214,10 @@ template <typename T> struct LamTab {
 // in shared memory, and the cluster adds the CTAs' partials through
 // distributed shared memory (double-buffered, one cluster barrier per block).
 // Deterministic order.
-template <typename T, int CP, bool TAB>
+template <int CP, bool TAB>
 __global__ void __launch_bounds__(512)
 k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const RingInfo* __restrict__ rings,
-                    const C2<T>* __restrict__ etab, const RecCoef<T>* __restrict__ coef_c,
+                    const C2<T>* __restrict__ etab, const double* __restrict__ coef_c,
                     const double* __restrict__ coef_p, const int* __restrict__ lc_tab,
                     const double* __restrict__ mu0_tab, const double* __restrict__ mu1_tab, int lmax,
                     int npair, int nring, long long nspec, long long nalm, int b0, int nb, int use_w,
@@ -218,7 +225,7 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
   using V = C2<T>;
   constexpr int C2N = 2 * CP;
   constexpr int CPL = LaneTile<C2N>::CPL, LPL = LaneTile<C2N>::LPL, NCQ = C2N / CPL;
-  constexpr int MS = MuStride<T>::v;
+  constexpr int MS = kMuStride;
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
   const int nthr = blockDim.x, nwarp = nthr >> 5;
@@ -231,7 +238,7 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
   T* sG = reinterpret_cast<T*>(smem_raw);      // [nthr][2][C2N]  S, A
   T* sMu = sG + (size_t)nthr * 2 * C2N;        // [nthr][MS]; warp w's [LB][C2N] partials at row 32 w
   T* sC = sMu + (size_t)nthr * MS;             // [2][LB][C2N]
-  RecCoef<T>* sCz = reinterpret_cast<RecCoef<T>*>(sC + 2 * LB * C2N);  // [2][LB] c_l of this and the next block
+  double* sCz = reinterpret_cast<double*>(sC + 2 * LB * C2N);  // [2][LB] c_l of this and the next block
 
   double z = 0.0, s0 = 0.0, s1 = 0.0;
   int lc = INT_MAX;
@@ -266,10 +273,10 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
   const long long base = alm_base(lmax, m);
   const int lq = lane / NCQ, cq = lane % NCQ;
   const int l0 = lq * LPL, c0 = cq * CPL;
-  Recur<T> rc;
+  RecurD rc;
   rc.start(z, s0, s1);
   int buf = 0;
-  if (t < LB) sCz[t] = (m + t <= lmax) ? coef_c[base + m + t] : RecCoef<T>{};
+  if (t < LB) sCz[t] = (m + t <= lmax) ? coef_c[base + m + t] : 0.0;
   // TAB: this warp's group rows (32 coalesced 128-byte rows per block),
   // loaded one block ahead so the loads are in flight during the contraction
   // and the reductions of the block before
@@ -290,18 +297,14 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
   }
   __syncthreads();
   for (int lb0 = m; lb0 <= lmax; lb0 += LB) {
-    const RecCoef<T>* cz = sCz + buf * LB;
+    const double* cz = sCz + buf * LB;
     // --- recurrence: LB steps of mu_l = c_l z mu_{l-1} - mu_{l-2} ---
     T* myMu = sMu + (size_t)t * MS;
     if constexpr (TAB) {
 #pragma unroll
       for (int i4 = 0; i4 < LB; i4 += 4) {
-        if constexpr (sizeof(T) == 4) {
-          *reinterpret_cast<float4*>(myMu + i4) = make_float4(nxt[i4], nxt[i4 + 1], nxt[i4 + 2], nxt[i4 + 3]);
-        } else {
-          *reinterpret_cast<double2*>(myMu + i4) = make_double2(nxt[i4], nxt[i4 + 1]);
-          *reinterpret_cast<double2*>(myMu + i4 + 2) = make_double2(nxt[i4 + 2], nxt[i4 + 3]);
-        }
+        *reinterpret_cast<double2*>(myMu + i4) = make_double2(nxt[i4], nxt[i4 + 1]);
+        *reinterpret_cast<double2*>(myMu + i4 + 2) = make_double2(nxt[i4 + 2], nxt[i4 + 3]);
       }
 #pragma unroll
       for (int i = 0; i < LB; ++i) {
@@ -314,12 +317,8 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
         T v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) v[u] = rc.step(cz[i4 + u], lb0 + i4 + u, lc);
-        if constexpr (sizeof(T) == 4) {
-          *reinterpret_cast<float4*>(myMu + i4) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
-          *reinterpret_cast<double2*>(myMu + i4) = make_double2(v[0], v[1]);
-          *reinterpret_cast<double2*>(myMu + i4 + 2) = make_double2(v[2], v[3]);
-        }
+        *reinterpret_cast<double2*>(myMu + i4) = make_double2(v[0], v[1]);
+        *reinterpret_cast<double2*>(myMu + i4 + 2) = make_double2(v[2], v[3]);
       }
     } else {
 #pragma unroll
@@ -372,7 +371,7 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
     // c_l of the next block, into the other half of the double buffer
     if (t < LB) {
       const int l = lb0 + LB + t;
-      sCz[(buf ^ 1) * LB + t] = (l <= lmax) ? coef_c[base + l] : RecCoef<T>{};
+      sCz[(buf ^ 1) * LB + t] = (l <= lmax) ? coef_c[base + l] : 0.0;
     }
     // --- cluster reduction; CTA r writes its share of the block ---
     cluster.sync();
@@ -397,225 +396,6 @@ k_legendre_analysis(const C2<T>* __restrict__ spec, T* __restrict__ alm, const R
 }
 
 // ---------------------------------------------------------------------------
-// analysis with the roles split (FP32 plans recomputing lambda)
-// ---------------------------------------------------------------------------
-// The same sums as k_legendre_analysis, but the first half of the CTA's
-// threads (producers, one chain each) only run the FP64 recurrence, writing
-// each block of LB values of mu into one of two shared-memory slots, and the
-// second half (consumers, consumer i serving producer i's chain) contract the
-// blocks, add the warps' and the cluster's partial sums and write alm.  The
-// producers do not wait for the sums, so the FP64 pipe is not left idle
-// while a CTA contracts and reduces.
-//   producer -> consumer: mbarrier full[slot], one arrival per producer,
-//     waited with a time limit;
-//   among the consumers: named barrier 1;
-//   slot reuse and the cluster sums: every thread takes one cluster-barrier
-//     phase per block -- consumers once their block's partials are written,
-//     producers for block b just before they write block b + 2 into b's
-//     slot (the phase that frees it) -- and one more at the end.
-// Deterministic order, as the one-role kernel.
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// true once the phase of `bar` with this parity has completed; false after 1 s
-__device__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
-  if (mbar_test(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  for (unsigned i = 1; i < (1u << 31); ++i) {
-    if (mbar_test(bar, parity)) return true;
-    if ((i & 63u) == 0 && global_ns() - t0 > 1000000000ull) break;
-  }
-  return false;
-}
-
-template <int CP>
-size_t analysis_ws_smem(int nch) {
-  constexpr int C2N = 2 * CP;
-  return 32 + sizeof(float) * ((size_t)nch * 2 * C2N + 2 * (size_t)nch * MuStride<float>::v + 2 * LB * C2N);
-}
-
-template <int CP>
-__global__ void __launch_bounds__(1024)
-k_legendre_analysis_ws(const float2* __restrict__ spec, float* __restrict__ alm, const RingInfo* __restrict__ rings,
-                       const float2* __restrict__ etab, const float2* __restrict__ coef_c,
-                       const double* __restrict__ coef_p, const int* __restrict__ lc_tab,
-                       const double* __restrict__ mu0_tab, const double* __restrict__ mu1_tab, int lmax,
-                       int npair, int nring, long long nspec, long long nalm, int b0, int nb, int use_w,
-                       double mfac, int* __restrict__ status) {
-  using T = float;
-  using V = float2;
-  constexpr int C2N = 2 * CP;
-  constexpr int CPL = LaneTile<C2N>::CPL, LPL = LaneTile<C2N>::LPL, NCQ = C2N / CPL;
-  constexpr int MS = MuStride<T>::v;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int crank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
-  const int nch = blockDim.x >> 1;  // chains of the CTA = producer threads = consumer threads
-  const int t = threadIdx.x, lane = t & 31;
-  const bool producer = t < nch;
-  const int ct = producer ? t : t - nch;  // the chain this thread serves
-  const int cw = ct >> 5, nw = nch >> 5;  // its warp among its role's warps
-  const int m = blockIdx.y;
-  const int p = (cw * csize + crank) * 32 + lane;
-  const bool active = p < npair;
-
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);  // [2]
-  T* sG = reinterpret_cast<T*>(smem_raw + 32);              // [nch][2][C2N]  S, A
-  T* sMu = sG + (size_t)nch * 2 * C2N;                      // [2][nch][MS]; a consumer warp's partials in its rows
-  T* sC = sMu + (size_t)2 * nch * MS;                       // [2][LB][C2N]
-
-  double z = 0.0, s0 = 0.0, s1 = 0.0;
-  int lc = INT_MAX;
-  if (active) {
-    const long long ci = (long long)m * npair + p;
-    z = rings[p].z;
-    lc = lc_tab[ci];
-    s0 = mu0_tab[ci];
-    s1 = mu1_tab[ci];
-    if (lc > lmax) lc = INT_MAX;
-  }
-  if (producer) {  // the chain's S and A coefficients, as in the one-role kernel
-    T* g = sG + (size_t)ct * 2 * C2N;
-    if (active) {
-      const int ys = (p == npair - 1) ? -1 : nring - 1 - p;
-      const RingInfo Rn = rings[p];
-      for (int c = 0; c < CP; ++c) {
-        V gn = cmk<V>(0, 0), gs = cmk<V>(0, 0);
-        if (c < nb && lc != INT_MAX) {
-          gn = ring_coef<T>(spec, etab, Rn, m, b0 + c, nspec, use_w);
-          if (ys >= 0) gs = ring_coef<T>(spec, etab, rings[ys], m, b0 + c, nspec, use_w);
-        }
-        const V S = cadd(gn, gs), A = csub(gn, gs);
-        g[2 * c] = S.x;
-        g[2 * c + 1] = S.y;
-        g[C2N + 2 * c] = A.x;
-        g[C2N + 2 * c + 1] = A.y;
-      }
-    } else {
-      for (int c = 0; c < 2 * C2N; ++c) g[c] = (T)0;
-    }
-  }
-  if (t == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[0])), "r"(nch));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[1])), "r"(nch));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();  // the last barrier of all the CTA's threads before the roles part
-
-  const long long base = alm_base(lmax, m);
-  const int nblk = (lmax - m) / LB + 1;
-  if (producer) {
-    // ---- the recurrence, block by block into slot b mod 2
-    const float2* cl = coef_c + base;
-    Recur<float> rc;
-    rc.start(z, s0, s1);
-    for (int b = 0; b < nblk; ++b) {
-      const int lb0 = m + b * LB, slot = b & 1;
-      if (b >= 2) cluster.sync();  // phase b - 2: every consumer is done with block b - 2, which used this slot
-      T* myMu = sMu + ((size_t)slot * nch + ct) * MS;
-      if (__any_sync(0xffffffffu, lc < lb0 + LB)) {
-#pragma unroll
-        for (int i4 = 0; i4 < LB; i4 += 4) {
-          float2 c4[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) c4[u] = (lb0 + i4 + u <= lmax) ? cl[lb0 + i4 + u] : make_float2(0.f, 0.f);
-          T v[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) v[u] = rc.step(c4[u], lb0 + i4 + u, lc);
-          *reinterpret_cast<float4*>(myMu + i4) = make_float4(v[0], v[1], v[2], v[3]);
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < LB; i += 4) *reinterpret_cast<float4*>(myMu + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[slot])) : "memory");
-    }
-    for (int b = nblk > 2 ? nblk - 2 : 0; b < nblk; ++b) cluster.sync();  // the phases of the last blocks
-  } else {
-    // ---- contraction and sums
-    const int lq = lane / NCQ, cq = lane % NCQ;
-    const int l0 = lq * LPL, c0 = cq * CPL;
-    bool timed_out = false;
-    for (int b = 0; b < nblk; ++b) {
-      const int lb0 = m + b * LB, slot = b & 1;
-      const bool ok = mbar_wait_bounded(&full[slot], (uint32_t)(b >> 1) & 1u);
-      if (!ok) timed_out = true;
-      T* muS = sMu + (size_t)slot * nch * MS;
-      T acc[LPL][CPL];
-#pragma unroll
-      for (int a = 0; a < LPL; ++a)
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) acc[a][c] = (T)0;
-      if (__all_sync(0xffffffffu, ok) && __any_sync(0xffffffffu, lc < lb0 + LB)) {
-        const T* muw = muS + (size_t)(cw * 32) * MS + l0;
-        const T* gw = sG + (size_t)(cw * 32) * 2 * C2N + c0;
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) {
-          T mv[LPL], gsv[CPL], gav[CPL];
-#pragma unroll
-          for (int a = 0; a < LPL; ++a) mv[a] = muw[(size_t)j * MS + a];
-#pragma unroll
-          for (int c = 0; c < CPL; ++c) {
-            gsv[c] = gw[(size_t)j * 2 * C2N + c];
-            gav[c] = gw[(size_t)j * 2 * C2N + C2N + c];
-          }
-#pragma unroll
-          for (int a = 0; a < LPL; ++a) {
-            const bool odd = ((l0 + a) & 1) != 0;
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) acc[a][c] = fma(mv[a], odd ? gav[c] : gsv[c], acc[a][c]);
-          }
-        }
-      }
-      // this warp's partials over its own 32 mu rows of the slot, which only it has read
-      T* wp = muS + (size_t)(cw * 32) * MS;
-      __syncwarp();
-#pragma unroll
-      for (int a = 0; a < LPL; ++a)
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) wp[(l0 + a) * C2N + c0 + c] = acc[a][c];
-      asm volatile("bar.sync 1, %0;" ::"r"(nch) : "memory");  // the consumers' partials are in
-      T* cpart = sC + slot * LB * C2N;
-      for (int o = ct; o < LB * C2N; o += nch) {
-        T s = (T)0;
-        for (int w = 0; w < nw; ++w) s += muS[(size_t)(w * 32) * MS + o];
-        cpart[o] = s;
-      }
-      cluster.sync();  // phase b
-      {
-        const int nout = LB * C2N;
-        const int per = (nout + csize - 1) / csize;
-        const int q_end = min(nout, (crank + 1) * per);
-        for (int q = crank * per + ct; q < q_end; q += nch) {
-          const int part = q & 1, li = (q >> 1) % LB, bb = (q >> 1) / LB;
-          const int l = lb0 + li;
-          if (l > lmax || bb >= nb) continue;
-          const int o = li * C2N + 2 * bb + part;
-          T s = (T)0;
-          for (int r = 0; r < csize; ++r) s += cluster.map_shared_rank(cpart, r)[o];
-          alm[((long long)(b0 + bb) * nalm + base + l) * 2 + part] =
-              (T)(coef_p[base + l] * (m > 0 ? mfac : 1.0) * (double)s);
-        }
-      }
-    }
-    if (timed_out) atomicExch(status, (int)HPX_ERR_TIMEOUT);
-  }
-  cluster.sync();  // peers may still read this CTA's partials
-}
-
-// ---------------------------------------------------------------------------
 // synthesis
 // ---------------------------------------------------------------------------
 // One thread per chain (m, pair): E_m = sum over even l - m of a_lm lambda_lm,
@@ -623,18 +403,17 @@ k_legendre_analysis_ws(const float2* __restrict__ spec, float* __restrict__ alm,
 // F_m(y') = E - O on its mirror (Eq. 24 before the ring transform).  The
 // block's coefficients (pre-multiplied by P_l) are broadcast from shared
 // memory; mu comes from the recurrence, or from the lambda table when TAB.
-template <typename T, int CP, bool TAB>
+template <int CP, bool TAB>
 __global__ void __launch_bounds__(128)
 k_legendre_synthesis(const T* __restrict__ alm, C2<T>* __restrict__ F, const RingInfo* __restrict__ rings,
-                     const RecCoef<T>* __restrict__ coef_c, const float* __restrict__ coef_pf,
-                     const double* __restrict__ coef_p, const int* __restrict__ lc_tab,
+                     const double* __restrict__ coef_c, const double* __restrict__ coef_p, const int* __restrict__ lc_tab,
                      const double* __restrict__ mu0_tab, const double* __restrict__ mu1_tab, int lmax,
                      int mmax, int npair, int nring, long long nalm, int b0, int nb, const LamTab<T> tb,
                      double mfac) {
   using V = C2<T>;
   constexpr int C2N = 2 * CP;
   __shared__ __align__(16) T sA[LB][C2N];
-  __shared__ RecCoef<T> sCz[LB];
+  __shared__ double sCz[LB];
   __shared__ int sMinLc;
   const int m = blockIdx.y, t = threadIdx.x, nthr = blockDim.x;
   const int p = blockIdx.x * nthr + t;
@@ -658,7 +437,7 @@ k_legendre_synthesis(const T* __restrict__ alm, C2<T>* __restrict__ F, const Rin
 #pragma unroll
   for (int c = 0; c < C2N; ++c) accE[c] = accO[c] = (T)0;
   const long long base = alm_base(lmax, m);
-  Recur<T> rc;
+  RecurD rc;
   rc.start(z, s0, s1);
   if (lstart <= lmax) {
     for (int lb0 = m + ((lstart - m) / LB) * LB; lb0 <= lmax; lb0 += LB) {
@@ -668,12 +447,11 @@ k_legendre_synthesis(const T* __restrict__ alm, C2<T>* __restrict__ F, const Rin
         T v = (T)0;
         if (l <= lmax && bb < nb && !(m == 0 && part == 1)) {
           const T a = alm[((long long)(b0 + bb) * nalm + base + l) * 2 + part];
-          if constexpr (sizeof(T) == 4) v = coef_pf[base + l] * (m > 0 ? (float)mfac : 1.0f) * a;
-          else v = (T)(coef_p[base + l] * (m > 0 ? mfac : 1.0) * (double)a);
+          v = coef_p[base + l] * (m > 0 ? mfac : 1.0) * a;
         }
         sA[li][c] = v;
       }
-      if (t < LB) sCz[t] = (lb0 + t <= lmax) ? coef_c[base + lb0 + t] : RecCoef<T>{};
+      if (t < LB) sCz[t] = (lb0 + t <= lmax) ? coef_c[base + lb0 + t] : 0.0;
       __syncthreads();
       // a warp whose chains all start after this block has nothing to add
       if (TAB && __any_sync(0xffffffffu, lc < lb0 + LB)) {
@@ -742,24 +520,14 @@ static void analysis_shape(int npair, int* nthr, int* csize) {
   }
 }
 
-template <typename T>
-static LamTab<T> lam_tab(const hpx_plan_s* p) {
-  LamTab<T> tb;
-  tb.tab = static_cast<const T*>(p->d_tab);
-  tb.off = p->d_tab_off;
-  tb.lstart = p->d_tab_lstart;
-  tb.ngroup = p->ngroup;
-  return tb;
-}
-
-template <typename T, int CP, bool TAB>
+template <int CP, bool TAB>
 static cudaError_t launch_analysis_cp(const hpx_plan_s* p, T* alm, bool use_w, double mfac, cudaStream_t s,
                                       int* nlaunch) {
   using V = C2<T>;
   int nthr, csize;
   analysis_shape(p->npair, &nthr, &csize);
-  const size_t smem = analysis_smem<T, CP>(nthr);
-  cudaError_t e = allow_max_smem(k_legendre_analysis<T, CP, TAB>);
+  const size_t smem = analysis_smem<CP>(nthr);
+  cudaError_t e = allow_max_smem(k_legendre_analysis<CP, TAB>);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(csize, p->mmax + 1, 1);
@@ -775,8 +543,8 @@ static cudaError_t launch_analysis_cp(const hpx_plan_s* p, T* alm, bool use_w, d
   cfg.numAttrs = 1;
   for (int b0 = 0; b0 < p->nbatch; b0 += CP) {
     const int nb = (p->nbatch - b0) < CP ? (p->nbatch - b0) : CP;
-    e = cudaLaunchKernelEx(&cfg, k_legendre_analysis<T, CP, TAB>, (const V*)p->d_spec, alm,
-                           (const RingInfo*)p->d_ring, (const V*)p->d_etab, rec_coefs<T>(p),
+    e = cudaLaunchKernelEx(&cfg, k_legendre_analysis<CP, TAB>, (const V*)p->d_spec, alm,
+                           (const RingInfo*)p->d_ring, (const V*)p->d_etab, (const double*)p->d_coef_c,
                            (const double*)p->d_coef_p, (const int*)p->d_lc, (const double*)p->d_mu0,
                            (const double*)p->d_mu1, p->lmax, p->npair, p->nring, p->nspec, p->nalm, b0, nb,
                            use_w ? 1 : 0, lam_tab<T>(p), mfac);
@@ -786,28 +554,26 @@ static cudaError_t launch_analysis_cp(const hpx_plan_s* p, T* alm, bool use_w, d
   return cudaGetLastError();
 }
 
-template <typename T, int CP>
+template <int CP>
 static cudaError_t launch_analysis_sel(const hpx_plan_s* p, T* alm, bool use_w, double mfac, cudaStream_t s,
                                        int* nlaunch) {
-  return p->d_tab ? launch_analysis_cp<T, CP, true>(p, alm, use_w, mfac, s, nlaunch)
-                  : launch_analysis_cp<T, CP, false>(p, alm, use_w, mfac, s, nlaunch);
+  return p->d_tab ? launch_analysis_cp<CP, true>(p, alm, use_w, mfac, s, nlaunch)
+                  : launch_analysis_cp<CP, false>(p, alm, use_w, mfac, s, nlaunch);
 }
 
-template <typename T>
 static int pick_cp(const hpx_plan_s* p) {
   int nthr, csize;
   analysis_shape(p->npair, &nthr, &csize);
-  const int cmax = sizeof(T) == 4 ? 16 : 8;
+  const int cmax = 8;
   int cp = 1;
   while (cp < p->nbatch && cp < cmax) cp *= 2;
   auto fits = [&](int c) {
     size_t sm = 0;
     switch (c) {
-      case 1: sm = analysis_smem<T, 1>(nthr); break;
-      case 2: sm = analysis_smem<T, 2>(nthr); break;
-      case 4: sm = analysis_smem<T, 4>(nthr); break;
-      case 8: sm = analysis_smem<T, 8>(nthr); break;
-      default: sm = analysis_smem<T, 16>(nthr); break;
+      case 1: sm = analysis_smem<1>(nthr); break;
+      case 2: sm = analysis_smem<2>(nthr); break;
+      case 4: sm = analysis_smem<4>(nthr); break;
+      default: sm = analysis_smem<8>(nthr); break;
     }
     return sm <= 200 * 1024;
   };
@@ -815,95 +581,18 @@ static int pick_cp(const hpx_plan_s* p) {
   return cp;
 }
 
-// The split-role analysis (FP32, lambda recomputed): clusters as for the
-// one-role kernel, twice the threads (producers and consumers).
-template <int CP>
-static cudaError_t launch_analysis_ws_cp(const hpx_plan_s* p, float* alm, bool use_w, double mfac, cudaStream_t s,
-                                         int* nlaunch) {
-  int nthr, csize;
-  analysis_shape(p->npair, &nthr, &csize);
-  const size_t smem = analysis_ws_smem<CP>(nthr);
-  cudaError_t e = allow_max_smem(k_legendre_analysis_ws<CP>);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(csize, p->mmax + 1, 1);
-  cfg.blockDim = dim3(2 * nthr, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = csize;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  for (int b0 = 0; b0 < p->nbatch; b0 += CP) {
-    const int nb = (p->nbatch - b0) < CP ? (p->nbatch - b0) : CP;
-    e = cudaLaunchKernelEx(&cfg, k_legendre_analysis_ws<CP>, (const float2*)p->d_spec, alm,
-                           (const RingInfo*)p->d_ring, (const float2*)p->d_etab, (const float2*)p->d_coef_cf,
-                           (const double*)p->d_coef_p, (const int*)p->d_lc, (const double*)p->d_mu0,
-                           (const double*)p->d_mu1, p->lmax, p->npair, p->nring, p->nspec, p->nalm, b0, nb,
-                           use_w ? 1 : 0, mfac, p->d_status);
-    if (e != cudaSuccess) return e;
-    ++*nlaunch;
-  }
-  return cudaGetLastError();
-}
-
-// Channels per launch of the split-role analysis: the largest power of two
-// up to cap with which two CTAs fit an SM (0 if none).  With one CTA per SM
-// (512 chains per CTA at Nside 2048, or wide channel groups) every cluster
-// barrier idles the SM's FP64 pipe, and the one-role kernel, whose CTAs
-// share SMs with other clusters', is faster (252 against 295 ms at Nside
-// 2048 / lmax 6143 / 4 channels).
-static int pick_cp_ws(int npair, int cap) {
-  int nthr, csize;
-  analysis_shape(npair, &nthr, &csize);
-  if (nthr > 256) return 0;
-  for (int cp = cap; cp >= 1; cp /= 2) {
-    size_t sm = 0;
-    switch (cp) {
-      case 1: sm = analysis_ws_smem<1>(nthr); break;
-      case 2: sm = analysis_ws_smem<2>(nthr); break;
-      case 4: sm = analysis_ws_smem<4>(nthr); break;
-      case 8: sm = analysis_ws_smem<8>(nthr); break;
-      default: sm = analysis_ws_smem<16>(nthr); break;
-    }
-    if (sm <= 112 * 1024) return cp;
-  }
-  return 0;
-}
-
-template <typename T>
-cudaError_t launch_analysis(const hpx_plan_s* p, T* alm, bool use_w, double mfac, cudaStream_t s, int* nlaunch) {
-  if constexpr (sizeof(T) == 4) {
-    // FP32 recomputing lambda: the split-role kernel, unless its channel
-    // groups would need more launches (each reruns the recurrence)
-    if (!p->d_tab) {
-      const int cp_one = pick_cp<T>(p), cp_ws = pick_cp_ws(p->npair, cp_one);
-      if (cp_ws > 0 && (p->nbatch + cp_ws - 1) / cp_ws == (p->nbatch + cp_one - 1) / cp_one) {
-        switch (cp_ws) {
-          case 1: return launch_analysis_ws_cp<1>(p, alm, use_w, mfac, s, nlaunch);
-          case 2: return launch_analysis_ws_cp<2>(p, alm, use_w, mfac, s, nlaunch);
-          case 4: return launch_analysis_ws_cp<4>(p, alm, use_w, mfac, s, nlaunch);
-          case 8: return launch_analysis_ws_cp<8>(p, alm, use_w, mfac, s, nlaunch);
-          default: return launch_analysis_ws_cp<16>(p, alm, use_w, mfac, s, nlaunch);
-        }
-      }
-    }
-  }
-  switch (pick_cp<T>(p)) {
-    case 1: return launch_analysis_sel<T, 1>(p, alm, use_w, mfac, s, nlaunch);
-    case 2: return launch_analysis_sel<T, 2>(p, alm, use_w, mfac, s, nlaunch);
-    case 4: return launch_analysis_sel<T, 4>(p, alm, use_w, mfac, s, nlaunch);
-    case 8: return launch_analysis_sel<T, 8>(p, alm, use_w, mfac, s, nlaunch);
-    default:
-      if constexpr (sizeof(T) == 4) return launch_analysis_sel<T, 16>(p, alm, use_w, mfac, s, nlaunch);
-      else return launch_analysis_sel<T, 8>(p, alm, use_w, mfac, s, nlaunch);
+template <>
+cudaError_t launch_analysis<double>(const hpx_plan_s* p, double* alm, bool use_w, double mfac, cudaStream_t s,
+                                    int* nlaunch) {
+  switch (pick_cp(p)) {
+    case 1: return launch_analysis_sel<1>(p, alm, use_w, mfac, s, nlaunch);
+    case 2: return launch_analysis_sel<2>(p, alm, use_w, mfac, s, nlaunch);
+    case 4: return launch_analysis_sel<4>(p, alm, use_w, mfac, s, nlaunch);
+    default: return launch_analysis_sel<8>(p, alm, use_w, mfac, s, nlaunch);
   }
 }
 
-template <typename T, int CP, bool TAB>
+template <int CP, bool TAB>
 static cudaError_t launch_synthesis_cp(const hpx_plan_s* p, const T* alm, double mfac, cudaStream_t s,
                                        int* nlaunch) {
   using V = C2<T>;
@@ -911,8 +600,8 @@ static cudaError_t launch_synthesis_cp(const hpx_plan_s* p, const T* alm, double
   dim3 grid((p->npair + nthr - 1) / nthr, p->mmax + 1);
   for (int b0 = 0; b0 < p->nbatch; b0 += CP) {
     const int nb = (p->nbatch - b0) < CP ? (p->nbatch - b0) : CP;
-    k_legendre_synthesis<T, CP, TAB><<<grid, nthr, 0, s>>>(
-        alm, (V*)p->d_F, p->d_ring, rec_coefs<T>(p), p->d_coef_pf, p->d_coef_p, p->d_lc, p->d_mu0, p->d_mu1,
+    k_legendre_synthesis<CP, TAB><<<grid, nthr, 0, s>>>(
+        alm, (V*)p->d_F, p->d_ring, (const double*)p->d_coef_c, p->d_coef_p, p->d_lc, p->d_mu0, p->d_mu1,
         p->lmax, p->mmax, p->npair, p->nring, p->nalm, b0, nb, lam_tab<T>(p), mfac);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -921,26 +610,23 @@ static cudaError_t launch_synthesis_cp(const hpx_plan_s* p, const T* alm, double
   return cudaSuccess;
 }
 
-template <typename T, int CP>
+template <int CP>
 static cudaError_t launch_synthesis_sel(const hpx_plan_s* p, const T* alm, double mfac, cudaStream_t s,
                                         int* nlaunch) {
-  return p->d_tab ? launch_synthesis_cp<T, CP, true>(p, alm, mfac, s, nlaunch)
-                  : launch_synthesis_cp<T, CP, false>(p, alm, mfac, s, nlaunch);
+  return p->d_tab ? launch_synthesis_cp<CP, true>(p, alm, mfac, s, nlaunch)
+                  : launch_synthesis_cp<CP, false>(p, alm, mfac, s, nlaunch);
 }
 
-template <typename T>
-cudaError_t launch_synthesis(const hpx_plan_s* p, const T* alm, double mfac, cudaStream_t s, int* nlaunch) {
+template <>
+cudaError_t launch_synthesis<double>(const hpx_plan_s* p, const double* alm, double mfac, cudaStream_t s,
+                                     int* nlaunch) {
   int cp = 1;
-  const int cmax = sizeof(T) == 4 ? 16 : 8;
-  while (cp < p->nbatch && cp < cmax) cp *= 2;
+  while (cp < p->nbatch && cp < 8) cp *= 2;
   switch (cp) {
-    case 1: return launch_synthesis_sel<T, 1>(p, alm, mfac, s, nlaunch);
-    case 2: return launch_synthesis_sel<T, 2>(p, alm, mfac, s, nlaunch);
-    case 4: return launch_synthesis_sel<T, 4>(p, alm, mfac, s, nlaunch);
-    case 8: return launch_synthesis_sel<T, 8>(p, alm, mfac, s, nlaunch);
-    default:
-      if constexpr (sizeof(T) == 4) return launch_synthesis_sel<T, 16>(p, alm, mfac, s, nlaunch);
-      else return launch_synthesis_sel<T, 8>(p, alm, mfac, s, nlaunch);
+    case 1: return launch_synthesis_sel<1>(p, alm, mfac, s, nlaunch);
+    case 2: return launch_synthesis_sel<2>(p, alm, mfac, s, nlaunch);
+    case 4: return launch_synthesis_sel<4>(p, alm, mfac, s, nlaunch);
+    default: return launch_synthesis_sel<8>(p, alm, mfac, s, nlaunch);
   }
 }
 
@@ -952,14 +638,31 @@ __global__ void k_coef_pairs(const double* __restrict__ coef_c, float2* __restri
   }
 }
 
+__global__ void k_z_pairs(const RingInfo* __restrict__ rings, float2* __restrict__ zf, int npair) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= npair) return;
+  const Df d = df_of(rings[p].z);
+  zf[p] = make_float2(d.hi, d.lo);
+}
+
 cudaError_t build_recurrence_tables(hpx_plan_s* p, cudaStream_t s) {
   const int mb = (p->mmax + 1 + 127) / 128;
   k_lambda_mm_prefactor<<<mb, 128, 0, s>>>(p->mmax, p->d_cmm);
-  k_recurrence_coefs<<<mb, 128, 0, s>>>(p->lmax, p->mmax, p->d_coef_c, p->d_coef_p, p->d_coef_pf);
+  k_recurrence_coefs<<<mb, 128, 0, s>>>(p->lmax, p->mmax, p->d_coef_c, p->d_coef_p, p->d_coef_pp, p->d_coef_pf);
   const long long nb = (p->nalm + 255) / 256;
   k_coef_pairs<<<(unsigned)(nb < 4096 ? nb : 4096), 256, 0, s>>>(p->d_coef_c, p->d_coef_cf, p->nalm);
+  const int mode = tc_mode_of(p->dtype, p->flags);
+  const bool half = mode > 0 && p->dtype != HPX_F32_BF16 && p->dtype != HPX_F32_BF16X3;
+  const int sig = p->dtype == HPX_F64 ? kSigExp64 : half ? kSigExpHalf : kSigExp32;
+  if (p->d_lgrid) {
+    const size_t bytes = sizeof(int) * (size_t)(p->mmax + 1) * p->ngrid;
+    cudaError_t e = cudaMemsetAsync(p->d_lgrid, 0, bytes, s);
+    if (e != cudaSuccess) return e;
+    k_z_pairs<<<(p->npair + 127) / 128, 128, 0, s>>>(p->d_ring, p->d_zf, p->npair);
+  }
   k_chain_scan<<<dim3((p->npair + 127) / 128, p->mmax + 1), 128, 0, s>>>(
-      p->d_ring, p->d_cmm, p->d_coef_c, p->lmax, p->npair, p->d_lc, p->d_mu0, p->d_mu1);
+      p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, sig, p->d_lc, p->d_mu0, p->d_mu1, p->d_start,
+      p->d_lgrid, p->ngrid);
   return cudaGetLastError();
 }
 
@@ -986,32 +689,39 @@ __global__ void k_table_groups(const int* __restrict__ lc_tab, int lmax, int npa
 }
 
 // Rows of every group: the recurrence of the per-transform kernels (same
-// operations, same conversion), zero before a chain's start and for the
-// padding lanes of a group.
-template <typename T>
-__global__ void k_table_fill(const RingInfo* __restrict__ rings, const RecCoef<T>* __restrict__ coef_c,
-                             const int* __restrict__ lc_tab, const double* __restrict__ mu0_tab,
-                             const double* __restrict__ mu1_tab, const int* __restrict__ lstart,
-                             const long long* __restrict__ off, int lmax, int npair, int ngroup, T* tab) {
+// operations), zero before a chain's start and for the padding lanes of a
+// group.
+template <typename E>
+__global__ void k_table_fill(const RingInfo* __restrict__ rings, const double* __restrict__ coef_c,
+                             const float2* __restrict__ coef_cf, const int* __restrict__ lc_tab,
+                             const double* __restrict__ mu0_tab, const double* __restrict__ mu1_tab,
+                             const float4* __restrict__ start, const int* __restrict__ lgrid, int ngrid,
+                             const int* __restrict__ lstart,
+                             const long long* __restrict__ off, int lmax, int npair, int ngroup, E* tab) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   const int g = p >> 5;
   if (g >= ngroup) return;
   const int ls = lstart[(long long)m * ngroup + g];
-  T* out = tab + off[(long long)m * ngroup + g] + (p & 31);
+  E* out = tab + off[(long long)m * ngroup + g] + (p & 31);
   if (p >= npair) {
-    for (int l = ls; l <= lmax; ++l) out[(long long)(l - ls) * 32] = (T)0;
+    for (int l = ls; l <= lmax; ++l) out[(long long)(l - ls) * 32] = (E)0;
     return;
   }
-  const long long ci = (long long)m * npair + p;
-  const int lc = lc_tab[ci];
-  Recur<T> rc;
-  rc.start(rings[p].z, mu0_tab[ci], mu1_tab[ci]);
-  const long long base = alm_base(lmax, m);
-  for (int l = ls; l <= lmax; ++l) out[(long long)(l - ls) * 32] = rc.step(coef_c[base + l], l, lc);
+  if constexpr (sizeof(E) == 4) {
+    Chain ch = chain_at<1>(rings, coef_cf, lc_tab, start, lgrid, ngrid, lmax, npair, m, p);
+    for (int l = ls; l <= lmax; ++l) out[(long long)(l - ls) * 32] = ch.step(l);
+  } else {
+    const long long ci = (long long)m * npair + p;
+    const int lc = lc_tab[ci];
+    RecurD rc;
+    rc.start(rings[p].z, mu0_tab[ci], mu1_tab[ci]);
+    const long long base = alm_base(lmax, m);
+    for (int l = ls; l <= lmax; ++l) out[(long long)(l - ls) * 32] = rc.step(coef_c[base + l], l, lc);
+  }
 }
 
-template <typename T>
+template <typename E>
 cudaError_t build_lambda_table(hpx_plan_s* p, cudaStream_t s) {
   const int ng = (p->npair + 31) / 32;
   p->ngroup = ng;
@@ -1039,20 +749,16 @@ cudaError_t build_lambda_table(hpx_plan_s* p, cudaStream_t s) {
   p->tab_elems = acc;
   e = cudaMemcpy(p->d_tab_off, rows.data(), sizeof(long long) * nent, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return e;
-  e = cudaMalloc(&p->d_tab, sizeof(T) * (acc > 0 ? acc : 1));
+  e = cudaMalloc(&p->d_tab, sizeof(E) * (acc > 0 ? acc : 1));
   if (e != cudaSuccess) return e;
-  p->bytes += sizeof(T) * (acc > 0 ? acc : 1);
-  k_table_fill<T><<<dim3((ng * 32 + 127) / 128, p->mmax + 1), 128, 0, s>>>(
-      p->d_ring, rec_coefs<T>(p), p->d_lc, p->d_mu0, p->d_mu1, p->d_tab_lstart, p->d_tab_off, p->lmax, p->npair,
-      ng, static_cast<T*>(p->d_tab));
+  p->bytes += sizeof(E) * (acc > 0 ? acc : 1);
+  k_table_fill<E><<<dim3((ng * 32 + 127) / 128, p->mmax + 1), 128, 0, s>>>(
+      p->d_ring, p->d_coef_c, p->d_coef_cf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_lgrid, p->ngrid, p->d_tab_lstart,
+      p->d_tab_off, p->lmax, p->npair, ng, static_cast<E*>(p->d_tab));
   return cudaGetLastError();
 }
 
 template cudaError_t build_lambda_table<float>(hpx_plan_s*, cudaStream_t);
 template cudaError_t build_lambda_table<double>(hpx_plan_s*, cudaStream_t);
-template cudaError_t launch_analysis<float>(const hpx_plan_s*, float*, bool, double, cudaStream_t, int*);
-template cudaError_t launch_analysis<double>(const hpx_plan_s*, double*, bool, double, cudaStream_t, int*);
-template cudaError_t launch_synthesis<float>(const hpx_plan_s*, const float*, double, cudaStream_t, int*);
-template cudaError_t launch_synthesis<double>(const hpx_plan_s*, const double*, double, cudaStream_t, int*);
 
 }  // namespace hpx

@@ -150,7 +150,7 @@ static void plan_free(hpx_plan_s* p) {
     delete[] st;
   }
   void* ptrs[] = {p->d_ring, p->d_etab, p->d_btab, p->d_chirp, p->d_tw, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->d_coef_p,
-                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
+                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_coef_pp, p->d_lgrid, p->d_zf, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
                   p->d_tab, p->d_tab_off, p->d_tab_lstart, p->d_gt, p->d_status, p->d_at, p->d_achunk,
                   p->d_stab, p->d_stab_off, p->d_stab_lstart, p->d_tab_lo, p->d_stab_lo, p->d_bmax,
                   p->d_it_map, p->d_it_alm};
@@ -407,6 +407,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
   p->nring = 4 * nside - 1;
   p->w_max = 4.0 * 3.14159265358979323846 / (12.0 * (double)nside * (double)nside);
   p->npair = 2 * nside;
+  p->ngrid = (p->npair + 63) / 64;
   p->npix = 12LL * nside * nside;
   p->nalm = hpx_nalm(lmax, mmax);
   p->nspec = 6LL * nside * nside + 4LL * nside - 1;
@@ -435,6 +436,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
     p->bytes += bytes;
     return true;
   };
+  const bool f64 = dtype == HPX_F64;
   bool ok = alloc((void**)&p->d_ring, sizeof(RingInfo) * p->nring) &&
             alloc(&p->d_etab, cs * p->netab) && alloc(&p->d_btab, cs * p->nbtab) &&
             alloc(&p->d_chirp, cs * (size_t)nside * (nside - 1)) &&
@@ -442,10 +444,14 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
             alloc((void**)&p->d_cmm, sizeof(double) * (mmax + 1)) &&
             alloc((void**)&p->d_coef_c, sizeof(double) * p->nalm) &&
             alloc((void**)&p->d_coef_cf, sizeof(float2) * p->nalm) &&
-            alloc((void**)&p->d_coef_p, sizeof(double) * p->nalm) &&
+            (f64 ? alloc((void**)&p->d_coef_p, sizeof(double) * p->nalm)
+                 : alloc((void**)&p->d_coef_pp, sizeof(float2) * p->nalm)) &&
             alloc((void**)&p->d_coef_pf, sizeof(float) * p->nalm) &&
-            alloc((void**)&p->d_lc, sizeof(int) * nchain) && alloc((void**)&p->d_mu0, sizeof(double) * nchain) &&
-            alloc((void**)&p->d_mu1, sizeof(double) * nchain) &&
+            alloc((void**)&p->d_lc, sizeof(int) * nchain) &&
+            (f64 ? alloc((void**)&p->d_mu0, sizeof(double) * nchain) && alloc((void**)&p->d_mu1, sizeof(double) * nchain)
+                 : alloc((void**)&p->d_start, sizeof(float4) * nchain) &&
+                       alloc((void**)&p->d_lgrid, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
+                       alloc((void**)&p->d_zf, sizeof(float2) * p->npair)) &&
             alloc(&p->d_spec, cs * (size_t)nbatch * p->nspec) &&
             alloc(&p->d_F, cs * (size_t)nbatch * p->nring * (mmax + 1)) &&
             alloc((void**)&p->d_status, sizeof(int));
@@ -532,7 +538,8 @@ size_t hpx_plan_estimate_bytes(int nside, int lmax, int mmax, int nbatch, hpx_dt
   size_t b = sizeof(RingInfo) * nring + cs * netab + cs * (nbtab ? nbtab : 1) + cs * ((size_t)1 << (logm_max - 1)) +
              cs * (size_t)nside * (nside - 1) +
              sizeof(double) * (mmax + 1) + (3 * sizeof(double) + sizeof(float)) * nalm +
-             (sizeof(int) + 2 * sizeof(double)) * nchain + cs * (size_t)nbatch * nspec +
+             (sizeof(int) + 2 * sizeof(double)) * nchain +
+             (dtype == HPX_F64 ? 0 : sizeof(int) * (size_t)(mmax + 1) * ((npair + 63) / 64) + sizeof(float2) * npair) + cs * (size_t)nbatch * nspec +
              cs * (size_t)nbatch * nring * (mmax + 1);
   const size_t ngroup = (npair + 31) / 32;
   const int mode = tc_mode_of(dtype, flags);

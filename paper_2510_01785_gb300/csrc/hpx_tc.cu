@@ -381,33 +381,11 @@ k_pack_at(const float2* __restrict__ alm, const float* __restrict__ coef_pf, con
 // ---------------------------------------------------------------------------
 // plan-time lambda tables of the tensor-core stages
 // ---------------------------------------------------------------------------
-// The recurrence of every table: the FP32 plans' chain (Recur<float>, the
-// same steps as the CUDA-core kernels', so FP32 tables hold identical
-// values), from l = ls, restarted at the chain start lc with the stored
-// (mu_{lc-1}, mu_lc); zero before lc.  16-bit tables hold kLamScale mu: the
-// restart values scaled by that power of two scale every later value
-// exactly.
-struct Chain {
-  Recur<float> rc;
-  int lc;
-  const float2* c;
-  __device__ __forceinline__ float step(int l) { return rc.step(c[l], l, lc); }
-};
-template <typename E>
-__device__ __forceinline__ Chain chain_at(const RingInfo* rings, const float2* coef_cf, const int* lc_tab,
-                                          const double* mu0_tab, const double* mu1_tab, int lmax, int npair, int m,
-                                          int p) {
-  Chain ch;
-  ch.lc = INT_MAX;
-  ch.c = coef_cf + alm_base(lmax, m);
-  if (p < npair) {
-    const long long ci = (long long)m * npair + p;
-    constexpr double kS = sizeof(E) == 2 ? kLamScale : 1.0;
-    ch.lc = lc_tab[ci];
-    ch.rc.start(rings[p].z, kS * mu0_tab[ci], kS * mu1_tab[ci]);
-  }
-  return ch;
-}
+// Every table takes the FP32 plans' chain (Chain: the same steps as the
+// CUDA-core kernels', so FP32 tables hold identical values).  16-bit tables
+// hold kLamScale mu: start values scaled by that power of two scale every
+// later value exactly.
+template <typename E> __host__ __device__ constexpr int chain_scale() { return sizeof(E) == 2 ? (int)kLamScale : 1; }
 // A table value as a stored element and its remainder: hi the FP32 value
 // rounded to E, lo the remainder (exact in FP32) rounded to E; hi + lo is
 // within 2^-22 |value| for 16-bit E.  FP32 tables store the value alone.
@@ -439,10 +417,10 @@ __global__ void k_rtab_groups(const int* __restrict__ lc_tab, int lmax, int npai
 // (base > 0 when the table is built block by block through a staging buffer).
 template <typename E>
 __global__ void k_rtab_fill(const RingInfo* __restrict__ rings, const float2* __restrict__ coef_c,
-                            const int* __restrict__ lc_tab, const double* __restrict__ mu0_tab,
-                            const double* __restrict__ mu1_tab, const int* __restrict__ lstart,
+                            const int* __restrict__ lc_tab, const float4* __restrict__ start,
+                            const int* __restrict__ lstart,
                             const long long* __restrict__ off, int lmax, int npair, int ngroup, int m0,
-                            long long base, E* hi, E* lo) {
+                            long long base, const int* __restrict__ lgrid, int ngrid, E* hi, E* lo) {
   constexpr int KW = Elt<E>::kw;
   const int p = blockIdx.x * blockDim.x + threadIdx.x, m = m0 + blockIdx.y;
   const int g = p / KW;
@@ -450,7 +428,7 @@ __global__ void k_rtab_fill(const RingInfo* __restrict__ rings, const float2* __
   const long long mg = (long long)m * ngroup + g;
   const int ls = lstart[mg];
   const long long o = off[mg] - base + (p % KW);
-  Chain ch = chain_at<E>(rings, coef_c, lc_tab, mu0_tab, mu1_tab, lmax, npair, m, p);
+  Chain ch = chain_at<chain_scale<E>()>(rings, coef_c, lc_tab, start, lgrid, ngrid, lmax, npair, m, p);
   // rows before the warp's first chain start are zero: no recurrence there
   // (a group's warps are whole, so the early return above left all lanes)
   const int lw = min(__reduce_min_sync(0xffffffffu, ch.lc), lmax + 1);
@@ -487,10 +465,10 @@ __global__ void k_ctab_tiles(const int* __restrict__ lc_tab, int lmax, int npair
 
 template <typename E>
 __global__ void k_ctab_fill(const RingInfo* __restrict__ rings, const float2* __restrict__ coef_c,
-                            const int* __restrict__ lc_tab, const double* __restrict__ mu0_tab,
-                            const double* __restrict__ mu1_tab, const int* __restrict__ lstart,
+                            const int* __restrict__ lc_tab, const float4* __restrict__ start,
+                            const int* __restrict__ lstart,
                             const long long* __restrict__ off, int lmax, int npair, int nptile, int m0,
-                            long long base, E* hi, E* lo) {
+                            long long base, const int* __restrict__ lgrid, int ngrid, E* hi, E* lo) {
   constexpr int KW = Elt<E>::kw, V = 16 / (int)sizeof(E);  // values per 16-byte store
   const int p = blockIdx.x * blockDim.x + threadIdx.x, m = m0 + blockIdx.y;
   const int T = p >> 7;
@@ -500,7 +478,7 @@ __global__ void k_ctab_fill(const RingInfo* __restrict__ rings, const float2* __
   if (ls > lmax) return;
   const int lend = ls + ((lmax - ls) / KW + 1) * KW;  // end of the last block
   const long long o = off[mT] - base + (long long)(p & 127) * KW;
-  Chain ch = chain_at<E>(rings, coef_c, lc_tab, mu0_tab, mu1_tab, lmax, npair, m, p);
+  Chain ch = chain_at<chain_scale<E>()>(rings, coef_c, lc_tab, start, lgrid, ngrid, lmax, npair, m, p);
   // vectors wholly before the warp's first chain start are zero: no
   // recurrence there (a tile's warps are whole: the early returns above
   // take all 128 threads of a tile or none)
@@ -1534,15 +1512,16 @@ template <typename E>
 cudaError_t fill_row_table(hpx_plan_s* p, int m0, int nm, long long base, void* hi, void* lo, cudaStream_t s) {
   constexpr int KW = Elt<E>::kw;
   k_rtab_fill<E><<<dim3((p->ngroup * KW + 127) / 128, nm), 128, 0, s>>>(
-      p->d_ring, p->d_coef_cf, p->d_lc, p->d_mu0, p->d_mu1, p->d_tab_lstart, p->d_tab_off, p->lmax, p->npair,
-      p->ngroup, m0, base, static_cast<E*>(hi), static_cast<E*>(lo));
+      p->d_ring, p->d_coef_cf, p->d_lc, p->d_start, p->d_tab_lstart, p->d_tab_off, p->lmax, p->npair,
+      p->ngroup, m0, base, p->d_lgrid, p->ngrid, static_cast<E*>(hi), static_cast<E*>(lo));
   return cudaGetLastError();
 }
 template <typename E>
 cudaError_t fill_col_table(hpx_plan_s* p, int m0, int nm, long long base, void* hi, void* lo, cudaStream_t s) {
-  k_ctab_fill<E><<<dim3(p->nptile, nm), 128, 0, s>>>(p->d_ring, p->d_coef_cf, p->d_lc, p->d_mu0, p->d_mu1,
+  k_ctab_fill<E><<<dim3(p->nptile, nm), 128, 0, s>>>(p->d_ring, p->d_coef_cf, p->d_lc, p->d_start,
                                                      p->d_stab_lstart, p->d_stab_off, p->lmax, p->npair,
-                                                     p->nptile, m0, base, static_cast<E*>(hi), static_cast<E*>(lo));
+                                                     p->nptile, m0, base, p->d_lgrid, p->ngrid, static_cast<E*>(hi),
+                                                     static_cast<E*>(lo));
   return cudaGetLastError();
 }
 cudaError_t fill_table(hpx_plan_s* p, bool col, int m0, int nm, long long base, void* hi, void* lo,

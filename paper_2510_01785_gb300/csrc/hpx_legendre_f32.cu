@@ -487,6 +487,14 @@ k_legendre_synthesis_f32(const float2* __restrict__ alm, float2* __restrict__ F,
       put(0, q);
     }
     __syncwarp();
+    float nxa[TAB ? 8 : 1], nxb[TAB ? 8 : 1];
+    if constexpr (TAB) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        nxa[u] = rows.a(lb0 + u, lmax);
+        nxb[u] = rows.b(lb0 + u, lmax);
+      }
+    }
     for (; lb0 <= lmax; lb0 += LB, buf ^= 1) {
 #pragma unroll 1
       for (int i8 = 0; i8 < LB; i8 += 8) {
@@ -494,10 +502,20 @@ k_legendre_synthesis_f32(const float2* __restrict__ alm, float2* __restrict__ F,
         if (next) fetch(lb0 + LB, i8 / 8);
         float va[8], vb[8];
         if constexpr (TAB) {
+          // this group of 8 was loaded a group ago; the next one's loads go out
+          // (16 channels leave no registers for that)
+          constexpr bool AHEAD = CP < 16;
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            va[u] = rows.a(lb0 + i8 + u, lmax);
-            vb[u] = rows.b(lb0 + i8 + u, lmax);
+            va[u] = AHEAD ? nxa[u] : rows.a(lb0 + i8 + u, lmax);
+            vb[u] = AHEAD ? nxb[u] : rows.b(lb0 + i8 + u, lmax);
+          }
+          if constexpr (AHEAD) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              nxa[u] = rows.a(lb0 + i8 + 8 + u, lmax);
+              nxb[u] = rows.b(lb0 + i8 + 8 + u, lmax);
+            }
           }
         } else {
           ch.steps8(&sCz[buf][i8], lb0 + i8, va, vb);

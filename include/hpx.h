@@ -104,10 +104,10 @@ typedef enum {
 } hpx_status;
 
 /* Plan flags for hpx_plan_create_ex. */
-#define HPX_PLAN_LAMBDA_RECOMPUTE 0u /* lambda_lm recomputed by the FP64
-                                        recurrence inside every transform */
+#define HPX_PLAN_LAMBDA_RECOMPUTE 0u /* lambda_lm recomputed by the recurrence
+                                        inside every transform */
 #define HPX_PLAN_LAMBDA_TABLE 1u     /* lambda_lm generated once at plan time
-                                        by the same FP64 recurrence and kept
+                                        by the same recurrence and kept
                                         in device memory (the precomputed
                                         Legendre tensor of Sec. III-D/III-G);
                                         results are identical to the
@@ -151,17 +151,16 @@ typedef enum {
                                         the resident plan. */
 #define HPX_PLAN_LAMBDA_STREAM 16u   /* with the tensor-core path: no table
                                         is kept; every transform recomputes
-                                        lambda by the FP64 recurrence (Eq.
-                                        15-16), block of m by block, into two
-                                        device staging buffers on a second
-                                        stream, and each block is contracted
-                                        on the tensor cores once it is
-                                        filled, while the recurrence fills
-                                        the other buffer.  One recurrence
-                                        serves all channels of the transform,
-                                        so the cost hardly grows with nbatch.
-                                        Same results as the resident plan
-                                        (the same fill kernels).  Not with
+                                        lambda (Eq. 15-16).  Split-product
+                                        plans (HPX_F32, HPX_F32_BF16X3,
+                                        HPX_F32_FP16X3) generate it in shared
+                                        memory beside the products; the others
+                                        fill two device staging buffers, block
+                                        of m by block, on a second stream while
+                                        the tensor cores contract the other.
+                                        One recurrence serves up to 32 channels
+                                        (split products) or all of them.  Same
+                                        results as the resident plan.  Not with
                                         HPX_PLAN_LAMBDA_HOST. */
 
 /* Number of packed coefficients for (lmax, mmax). */

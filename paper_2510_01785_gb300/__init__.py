@@ -84,7 +84,7 @@ class Plan:
             raise ValueError("out_of_core and streamed exclude each other")
         h = ctypes.c_void_p()
         with torch.cuda.device(self.device):
-            if streamed:  # lambda recomputed per transform into staging slabs, tensor-core products
+            if streamed:  # lambda recomputed per transform, tensor-core products
                 check(lib().hpx_plan_create_stream(nside, lmax, mmax, nbatch, DTYPES[dtype],
                                                    _lib.HPX_PLAN_TC_TF32X3 if tf32x3 else 0, int(stage_bytes),
                                                    ctypes.byref(h)), "hpx_plan_create_stream")

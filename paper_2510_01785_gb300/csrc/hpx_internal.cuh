@@ -75,7 +75,13 @@ struct hpx_plan_s {
   int* d_lgrid;        // [mmax+1][ngrid] first l from which every chain of a 64-pair group has |mu| >= 2^-kGridExp
                        // and is past its start (lmax + 1 if some chain never is); FP32 plans
   int ngrid;           // 64-pair groups
+  int* d_gstart;       // [mmax+1][ngrid] earliest start of a group's chains
   float2* d_zf;        // [npair] z as a sum of two floats
+  // generated-lambda tensor-core stages (hpx_gen.cu)
+  int gen_parts;       // 0: not used; 2: streamed split-product plans; 3: FP32 analysis in three BF16 parts
+  int gen_nn;          // 3: N columns of the analysis products
+  int gen_ctas;        // CTAs of the analysis (one per SM)
+  float4* d_gen_state; // [gen_ctas][npair] chains between tiles
   void* d_spec;        // workspace [nbatch][nspec] C2<T>
   void* d_F;           // workspace [nbatch][nring][mmax+1] C2<T>
   void* d_io_map;      // device I/O buffers of the host-buffer entry points (lazy)
@@ -628,13 +634,22 @@ cudaError_t build_lambda_table(hpx_plan_s* p, cudaStream_t s);
 // (row and column, hi and for x3 lo parts) are built here too.
 int tc_columns(int nbatch, int cap);  // N of a tile for nbatch channels, at most cap per launch
 int tc_mode_of(int dtype, unsigned flags);  // 0 3xTF32, 1 one 16-bit product, 2 16-bit x3; -1 none
-size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mode, bool host_tables);
+size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mode, bool host_tables, bool streamed);
 cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s);
 int tc_channels_per_launch(const hpx_plan_s* p, bool synthesis);
 cudaError_t launch_pack_tc(hpx_plan_s* p, int b0, int nb, bool use_weight, cudaStream_t s);
 cudaError_t launch_tile_tc(hpx_plan_s* p, float* alm, int b0, int nb, double mfac, cudaStream_t s);
 cudaError_t launch_pack_at_tc(hpx_plan_s* p, const float* alm, int b0, int nb, double mfac, cudaStream_t s);
 cudaError_t launch_synthesis_tc(hpx_plan_s* p, int b0, int nb, cudaStream_t s);
+// lambda generated in the kernel (hpx_gen.cu): the analysis reads the packed
+// operand Gt (launch_pack_tc; launch_pack_gen for the FP32 plans, whose operand
+// buffers build_gen makes), the synthesis At, as the table tiles do
+cudaError_t build_gen(hpx_plan_s* p, int parts);
+size_t gen_extra_bytes_estimate(int nside, int mmax, int nbatch, int parts);
+int gen_parts_of(int nside, int nbatch, int dtype, unsigned flags);
+cudaError_t launch_pack_gen(hpx_plan_s* p, int b0, int nb, bool use_weight, cudaStream_t s);
+cudaError_t launch_gen_analysis(const hpx_plan_s* p, float* alm, double mfac, cudaStream_t s);
+cudaError_t launch_gen_synthesis(const hpx_plan_s* p, cudaStream_t s);
 void free_tc_host(hpx_plan_s* p);  // out-of-core resources (pinned tables, stream, events)
 
 }  // namespace hpx

@@ -104,11 +104,12 @@ __global__ void k_recurrence_coefs(int lmax, int mmax, double* coef_c, double* c
 // FP32 plans (lgrid given, zeroed before): also, per group of 64 pairs, the
 // largest over its chains of the first l past l_c at which |mu_l| >=
 // 2^-kGridExp (lmax + 1 where a chain never gets there; a plain FP32
-// recurrence finds it).
+// recurrence finds it), and in gstart (large before) the earliest l_c.
 __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* __restrict__ cmm,
                              const double* __restrict__ coef_c, const float2* __restrict__ coef_cf, int lmax,
                              int npair, int sig, int* lc_tab, double* mu0_tab, double* mu1_tab,
-                             float4* __restrict__ start, int* __restrict__ lgrid, int ngrid) {
+                             float4* __restrict__ start, int* __restrict__ lgrid, int* __restrict__ gstart,
+                             int ngrid) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (p >= npair) return;
@@ -177,7 +178,11 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
   const int left = npair - (p & ~31);
   const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
   lg = __reduce_max_sync(mask, lg);
-  if ((threadIdx.x & 31) == 0) atomicMax(lgrid + (long long)m * ngrid + (p >> 6), lg);
+  const int ls = __reduce_min_sync(mask, lc_tab[ci]);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(lgrid + (long long)m * ngrid + (p >> 6), lg);
+    atomicMin(gstart + (long long)m * ngrid + (p >> 6), ls);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -657,12 +662,13 @@ cudaError_t build_recurrence_tables(hpx_plan_s* p, cudaStream_t s) {
   if (p->d_lgrid) {
     const size_t bytes = sizeof(int) * (size_t)(p->mmax + 1) * p->ngrid;
     cudaError_t e = cudaMemsetAsync(p->d_lgrid, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_gstart, 0x7f, bytes, s);
     if (e != cudaSuccess) return e;
     k_z_pairs<<<(p->npair + 127) / 128, 128, 0, s>>>(p->d_ring, p->d_zf, p->npair);
   }
   k_chain_scan<<<dim3((p->npair + 127) / 128, p->mmax + 1), 128, 0, s>>>(
       p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, sig, p->d_lc, p->d_mu0, p->d_mu1, p->d_start,
-      p->d_lgrid, p->ngrid);
+      p->d_lgrid, p->d_gstart, p->ngrid);
   return cudaGetLastError();
 }
 

@@ -150,7 +150,8 @@ static void plan_free(hpx_plan_s* p) {
     delete[] st;
   }
   void* ptrs[] = {p->d_ring, p->d_etab, p->d_btab, p->d_chirp, p->d_tw, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->d_coef_p,
-                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_coef_pp, p->d_lgrid, p->d_zf, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
+                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_coef_pp, p->d_lgrid, p->d_gstart, p->d_zf,
+                  p->d_gen_state, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
                   p->d_tab, p->d_tab_off, p->d_tab_lstart, p->d_gt, p->d_status, p->d_at, p->d_achunk,
                   p->d_stab, p->d_stab_off, p->d_stab_lstart, p->d_tab_lo, p->d_stab_lo, p->d_bmax,
                   p->d_it_map, p->d_it_alm};
@@ -229,6 +230,24 @@ static cudaError_t run_analysis(hpx_plan_s* p, const void* map, void* alm, bool 
       e = staged(p, 1, s, [&](int* n) {
         *n = 1;
         return launch_tile_tc(p, static_cast<float*>(alm), 0, p->nbatch, mfac, s);
+      });
+    return e;
+  }
+  if (p->gen_parts == 3) {
+    // FP32 without tensor-core tables: the packs, then one launch that
+    // generates lambda and contracts it for all channel groups
+    const int cp = p->gen_nn / 4;
+    for (int b0 = 0; b0 < p->nbatch && e == cudaSuccess; b0 += cp) {
+      const int nb = p->nbatch - b0 < cp ? p->nbatch - b0 : cp;
+      e = staged(p, 4, s, [&](int* n) {
+        *n = 1;
+        return launch_pack_gen(p, b0, nb, weighted, s);
+      });
+    }
+    if (e == cudaSuccess)
+      e = staged(p, 1, s, [&](int* n) {
+        *n = 1;
+        return launch_gen_analysis(p, static_cast<float*>(alm), mfac, s);
       });
     return e;
   }
@@ -451,6 +470,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
             (f64 ? alloc((void**)&p->d_mu0, sizeof(double) * nchain) && alloc((void**)&p->d_mu1, sizeof(double) * nchain)
                  : alloc((void**)&p->d_start, sizeof(float4) * nchain) &&
                        alloc((void**)&p->d_lgrid, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
+                       alloc((void**)&p->d_gstart, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
                        alloc((void**)&p->d_zf, sizeof(float2) * p->npair)) &&
             alloc(&p->d_spec, cs * (size_t)nbatch * p->nspec) &&
             alloc(&p->d_F, cs * (size_t)nbatch * p->nring * (mmax + 1)) &&
@@ -492,6 +512,8 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
       !(flags & (HPX_PLAN_LAMBDA_HOST | HPX_PLAN_LAMBDA_STREAM)))
     e = dtype == HPX_F64 ? build_lambda_table<double>(p, s) : build_lambda_table<float>(p, s);
   if (e == cudaSuccess && (flags & HPX_PLAN_TENSOR_CORES)) e = build_tc(p, s);
+  if (e == cudaSuccess)
+    if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) e = build_gen(p, parts);
   if (e == cudaSuccess) e = dtype == HPX_F64 ? build_fft_tables<double>(p, s) : build_fft_tables<float>(p, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
@@ -539,18 +561,20 @@ size_t hpx_plan_estimate_bytes(int nside, int lmax, int mmax, int nbatch, hpx_dt
              cs * (size_t)nside * (nside - 1) +
              sizeof(double) * (mmax + 1) + (3 * sizeof(double) + sizeof(float)) * nalm +
              (sizeof(int) + 2 * sizeof(double)) * nchain +
-             (dtype == HPX_F64 ? 0 : sizeof(int) * (size_t)(mmax + 1) * ((npair + 63) / 64) + sizeof(float2) * npair) + cs * (size_t)nbatch * nspec +
+             (dtype == HPX_F64 ? 0 : 2 * sizeof(int) * (size_t)(mmax + 1) * ((npair + 63) / 64) + sizeof(float2) * npair) + cs * (size_t)nbatch * nspec +
              cs * (size_t)nbatch * nring * (mmax + 1);
   const size_t ngroup = (npair + 31) / 32;
   const int mode = tc_mode_of(dtype, flags);
+  if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) b += gen_extra_bytes_estimate(nside, mmax, nbatch, parts);
   if (flags & (HPX_PLAN_LAMBDA_HOST | HPX_PLAN_LAMBDA_STREAM))  // no resident table; two staging buffers
-    return b + sizeof(int) + tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, true);
-  if (mode > 0) return b + sizeof(int) + tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, false);
+    return b + sizeof(int) +
+           tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, true, (flags & HPX_PLAN_LAMBDA_STREAM) != 0);
+  if (mode > 0) return b + sizeof(int) + tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, false, false);
   if (flags & HPX_PLAN_LAMBDA_TABLE)  // upper bound: every (l, m, ring pair) stored
     b += rs * nalm * npair + (sizeof(int) + sizeof(long long)) * (size_t)(mmax + 1) * ngroup;
   if (flags & HPX_PLAN_TENSOR_CORES)  // row-table starts padded to the tile grid; column table; operands
     b += rs * (size_t)(mmax + 1) * ngroup * 32 * (kTcTile - 1) +
-         tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, false);
+         tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, false, false);
   return b + sizeof(int);
 }
 

@@ -35,184 +35,15 @@
 // memory and returns; its output rows are then left unwritten.
 #include <cuda.h>
 #include <cudaTypedefs.h>
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <climits>
 #include <vector>
 
-#include "hpx_internal.cuh"
+#include "hpx_tcgen05.cuh"
 
 namespace hpx {
 namespace {
-
-constexpr unsigned long long kWaitNs = 1000000000ull;  // 1 s per wait
-// 16-bit lambda tables hold 2^9 lambda (|lambda_lm| <= sqrt((2l+1)/4pi) < 64
-// for l < 25000, so 2^9 |lambda| < 2^15 stays in FP16 range), which keeps
-// the FP16 remainder parts of small values out of the subnormal range; the
-// epilogues multiply by 2^-9.
-constexpr double kLamScale = 512.0;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Wait for the phase of `bar` with the given parity.  Gives up (false) when
-// another thread of the CTA has raised the abort flag (if watch_abort) or
-// after kWaitNs, raising the flag itself.
-__device__ bool wait_phase(uint64_t* bar, uint32_t parity, volatile int* abort_flag, bool watch_abort) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  for (unsigned i = 1; i < (1u << 31); ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 63u) == 0) {
-      if (watch_abort && *abort_flag) return false;
-      if (global_ns() - t0 > kWaitNs) break;
-    }
-  }
-  *abort_flag = 1;
-  return false;
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const void* map, int c0, int c1, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_u32(dst)),
-      "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(smem_u32(bar))
-      : "memory");
-}
-// Shared-memory matrix descriptor of a K-major operand in the 128-byte
-// swizzle: rows of 128 bytes, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-__device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-// A operand in tensor memory (lane = row, one 32-bit column per K element)
-__device__ __forceinline__ void umma_tf32_ta(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
-      "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc));
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-// 16 consecutive accumulator columns of this warp's 32 TMEM lanes (complete
-// after tmem_wait_ld).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// 32 consecutive columns of this warp's 32 TMEM lanes, complete on return.
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
-      "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
-      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
-      "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
-      "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-// x rounded to the nearest TF32 value (ties away from zero): the 13 low
-// mantissa bits rounded into the upper 19.  Finite inputs of table and
-// spectrum magnitude only (no overflow to infinity can occur there).
-__device__ __forceinline__ float tf32_rn(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
-}
-// The part of x the tensor cores drop (they read the TF32 truncation of x),
-// exact in FP32, itself rounded to TF32.
-__device__ __forceinline__ float tf32_rem(float x) {
-  return tf32_rn(x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u));
-}
-__device__ __forceinline__ float4 tf32_rem4(float4 x) {
-  return make_float4(tf32_rem(x.x), tf32_rem(x.y), tf32_rem(x.z), tf32_rem(x.w));
-}
-
-// ---------------------------------------------------------------------------
-// operand element types
-// ---------------------------------------------------------------------------
-// float: FP32 tables and operands; the products are 3xTF32 with the
-//   remainders made in shared memory (mode 0).
-// __nv_bfloat16 / __half: 16-bit tables and operands (kind::f16 products,
-//   FP32 accumulation); the hi part, and for the x3 modes the lo part
-//   lo = x - hi rounded again, are stored (modes 1 and 2).
-// A row of any operand tile is 128 bytes: 32 floats or 64 16-bit values.
-template <typename E> struct Elt;
-template <> struct Elt<float> {
-  static constexpr int kw = 32;
-  static __device__ __forceinline__ float from_float(float v) { return v; }
-  static __device__ __forceinline__ float to_float(float v) { return v; }
-};
-template <> struct Elt<__nv_bfloat16> {
-  static constexpr int kw = 64;
-  static __device__ __forceinline__ __nv_bfloat16 from_float(float v) { return __float2bfloat16_rn(v); }
-  static __device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
-};
-template <> struct Elt<__half> {
-  static constexpr int kw = 64;
-  static __device__ __forceinline__ __half from_float(float v) { return __float2half_rn(v); }
-  static __device__ __forceinline__ float to_float(__half v) { return __half2float(v); }
-};
-
-// Operand value v (already scaled) into row n of a tile column: hi at row n,
-// and for x3 the remainder at row NN + n.
-template <typename E>
-__device__ __forceinline__ void put(E* col, int n, int NN, float v, bool x3) {
-  constexpr int KW = Elt<E>::kw;
-  const E h = Elt<E>::from_float(v);
-  col[(long long)n * KW] = h;
-  if (x3) col[(long long)(NN + n) * KW] = Elt<E>::from_float(v - Elt<E>::to_float(h));
-}
-
-// Power of two s with s * bound <= 2^14, from the channel's recorded largest
-// component |x| (bit pattern of a non-negative float) times sfac, so that
-// FP16 operands stay in range; 1 without a record (FP32 operands) or for an
-// all-zero channel.
-__device__ __forceinline__ float chan_scale(const unsigned* bmax, int b, float sfac) {
-  if (!bmax) return 1.f;
-  const float amax = __uint_as_float(bmax[b]) * sfac;
-  if (!(amax > 0.f) || !(amax < 3.0e38f)) return 1.f;
-  int e;
-  frexpf(amax, &e);  // amax < 2^e
-  return ldexpf(1.f, min(14 - e, 126));  // 2^126 at most, so that the scale and its inverse are normal
-}
 
 // Largest |component| of each channel b0 .. b0+nb-1 of x ([b][stride]
 // complex values, n per channel), as float bits, into bmax[b] (atomic max;
@@ -243,7 +74,7 @@ __global__ void k_absmax(const float2* __restrict__ x, long long n, long long st
 // nothing) G(y) = W_y X_y[m mod N] exp(-i m phi_0) as in the CUDA-core
 // analysis; row n < 2 CP holds part n%2 of S = G(north) + G(south) for channel
 // n/2, row 2 CP + n that of A = G(north) - G(south), times the channel's
-// scale; for x3 rows NN .. 2 NN - 1 hold the remainders.
+// scale; rows NN .. 2 NN - 1 (and 2 NN .. 3 NN - 1) hold the remainders.
 //
 // One CTA: group g (KW pairs) x kPackM consecutive m x kPackC channels.  The
 // spectra are read along m (kPackM consecutive bins of one ring and channel
@@ -253,21 +84,21 @@ __global__ void k_absmax(const float2* __restrict__ x, long long n, long long st
 // all the CTA's channels of it.
 constexpr int kPackM = 8, kPackC = 8;
 
-__host__ __device__ constexpr int pack_rows(bool x3) { return (x3 ? 8 : 4) * kPackC; }  // shared rows per m
+__host__ __device__ constexpr int pack_rows(int parts) { return 4 * kPackC * parts; }  // shared rows per m
 __host__ __device__ constexpr int pack_slab(int rows) { return rows * 128 + 16; }  // bytes; 16 against bank conflicts
 
-template <typename E>
+template <typename E, int PARTS>
 __global__ void __launch_bounds__(256)
 k_pack_gt(const float2* __restrict__ spec, const float2* __restrict__ etab, const RingInfo* __restrict__ rings,
           E* __restrict__ gt, int npair, int nring, int ngroup, long long nspec, int mmax, int NN, int b0, int nb,
-          int use_w, int x3, const unsigned* __restrict__ bmax, float sfac) {
+          int use_w, const unsigned* __restrict__ bmax, float sfac) {
   constexpr int KW = Elt<E>::kw;
   // dynamic shared memory only (the launch may raise its limit to the
   // device maximum): kPackM slabs, then the channel scales
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int g = blockIdx.x, m0 = blockIdx.y * kPackM, c0 = blockIdx.z * kPackC;
-  const int C2N = NN / 2, rb = x3 ? 2 * NN : NN;
-  const int rows = pack_rows(x3 != 0), slab = pack_slab(rows);
+  const int C2N = NN / 2, rb = PARTS * NN;
+  constexpr int rows = pack_rows(PARTS), slab = pack_slab(rows);
   float* csc = reinterpret_cast<float*>(smem_raw + kPackM * slab);
   if (threadIdx.x < kPackC) {
     const int c = c0 + threadIdx.x;
@@ -318,21 +149,25 @@ k_pack_gt(const float2* __restrict__ spec, const float2* __restrict__ etab, cons
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int r = (q >> 1) * 2 * kPackC + 2 * cl + (q & 1);  // S rows, then A rows
-        const E h = Elt<E>::from_float(v[q]);
-        T[r * KW] = h;
-        if (x3) T[(r + 4 * kPackC) * KW] = Elt<E>::from_float(v[q] - Elt<E>::to_float(h));
+        float x = v[q];  // each part the remainder of those before it
+#pragma unroll
+        for (int part = 0; part < PARTS; ++part) {
+          const E h = Elt<E>::from_float(x);
+          T[(r + 4 * kPackC * part) * KW] = h;
+          x -= Elt<E>::to_float(h);
+        }
       }
     }
   }
   __syncthreads();
-  // local row rr: part rr / (2 kPackC) (S hi, A hi, S lo, A lo) at operand
-  // row (A: + C2N) (lo: + NN) + 2 c0 + rr % (2 kPackC)
+  // local row rr: part rr / (2 kPackC) (S hi, A hi, S lo, A lo, ...) at operand
+  // row (A: + C2N) (+ NN per remainder) + 2 c0 + rr % (2 kPackC)
   for (int q = threadIdx.x; q < kPackM * rows * 8; q += blockDim.x) {
     const int ml = q / (rows * 8), rr = (q >> 3) % rows, ch = q & 7;
     const int m = m0 + ml;
     if (m > mmax) continue;
     const int part = rr / (2 * kPackC);
-    const int grow = ((part & 1) ? C2N : 0) + ((part & 2) ? NN : 0) + 2 * c0 + rr % (2 * kPackC);
+    const int grow = ((part & 1) ? C2N : 0) + (part >> 1) * NN + 2 * c0 + rr % (2 * kPackC);
     const uint4 val = *reinterpret_cast<const uint4*>(smem_raw + ml * slab + rr * 128 + ch * 16);
     *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(gt) +
                               (((long long)m * ngroup + g) * rb + grow) * 128 + ch * 16) = val;
@@ -828,7 +663,7 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         const uint32_t aL = smem_u32(sL(s)), aLlo = smem_u32(sLlo(s, b)), aB = smem_u32(sB(s)),
                        aBlo = smem_u32(sBlo(s));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {  // 32 bytes along K per instruction (8 tf32 or 16 16-bit values)
+        for (int j = 0; j < (MODE == 2 ? 0 : 4); ++j) {  // 32 bytes along K per instruction (8 tf32 or 16 16-bit values)
           const uint32_t off = 32u * j;
           if constexpr (MODE == 0) {
             umma_tf32(d, sdesc_sw128(aL + off), sdesc_sw128(aB + off), id2, j > 0 ? 1u : 0u);
@@ -838,10 +673,19 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
               umma_tf32(d, sdesc_sw128(aLlo + off), sdesc_sw128(aB + off), id1, 1u);
           } else {
             umma_f16(d, sdesc_sw128(aL + off), sdesc_sw128(aB + off), id1, j > 0 ? 1u : 0u);
-            if constexpr (MODE == 2) {
-              umma_f16(d, sdesc_sw128(aL + off), sdesc_sw128(aBlo + off), id1, 1u);
-              umma_f16(d, sdesc_sw128(aLlo + off), sdesc_sw128(aB + off), id1, 1u);
-            }
+          }
+        }
+        if constexpr (MODE == 2) {
+          // per half of the block the remainder of L first, then L against both
+          // parts of B (the generated tiles' order, hpx_gen.cu: few additions
+          // truncate at the sum's own magnitude, and L is read once for both)
+#pragma unroll
+          for (int j = 0; j < 4; j += 2) {
+            const uint32_t o0 = 32u * j, o1 = o0 + 32u;
+            umma_f16(d, sdesc_sw128(aLlo + o0), sdesc_sw128(aB + o0), id1, j > 0 ? 1u : 0u);
+            umma_f16(d, sdesc_sw128(aLlo + o1), sdesc_sw128(aB + o1), id1, 1u);
+            umma_f16_pair(d, sdesc_sw128(aL + o0), sdesc_sw128(aBlo + o0), sdesc_sw128(aB + o0), id1, 1u);
+            umma_f16_pair(d, sdesc_sw128(aL + o1), sdesc_sw128(aBlo + o1), sdesc_sw128(aB + o1), id1, 1u);
           }
         }
         umma_commit(&empty[s]);
@@ -1257,17 +1101,17 @@ struct TileRange {
   long long tbase;
 };
 
-template <int CP, typename E>
+template <int CP, typename E, int PARTS>
 cudaError_t pack_gt_cp(const hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream_t s) {
   static_assert(CP % kPackC == 0, "channel blocks");  // CP >= 8
-  const bool x3 = p->tc_mode == 2;
-  const size_t smem = (size_t)kPackM * pack_slab(pack_rows(x3)) + kPackC * sizeof(float);
-  cudaError_t e = allow_max_smem(k_pack_gt<E>);
+  constexpr size_t smem = (size_t)kPackM * pack_slab(pack_rows(PARTS)) + kPackC * sizeof(float);
+  cudaError_t e = allow_max_smem(k_pack_gt<E, PARTS>);
   if (e != cudaSuccess) return e;
   E* gt = (E*)p->d_gt + (long long)(b0 / CP) * p->gt_group_elems;  // the group's region
-  k_pack_gt<E><<<dim3(p->ngroup, (p->mmax + kPackM) / kPackM, CP / kPackC), 256, smem, s>>>(
-      (const float2*)p->d_spec, (const float2*)p->d_etab, p->d_ring, gt, p->npair, p->nring, p->ngroup,
-      p->nspec, p->mmax, 4 * CP, b0, nb, use_w ? 1 : 0, x3 ? 1 : 0, p->tc_mode ? p->d_bmax : nullptr, p->tc_sfac_a);
+  const int ngroup = p->gen_parts == 3 ? p->ngrid : p->ngroup;
+  k_pack_gt<E, PARTS><<<dim3(ngroup, (p->mmax + kPackM) / kPackM, CP / kPackC), 256, smem, s>>>(
+      (const float2*)p->d_spec, (const float2*)p->d_etab, p->d_ring, gt, p->npair, p->nring, ngroup,
+      p->nspec, p->mmax, 4 * CP, b0, nb, use_w ? 1 : 0, p->tc_mode ? p->d_bmax : nullptr, p->tc_sfac_a);
   return cudaGetLastError();
 }
 
@@ -1308,9 +1152,12 @@ cudaError_t tile_cp(const hpx_plan_s* p, float* out, int b0, int nb, double mfac
 // Dispatch on the plan's operand type (float for mode 0, else 16-bit).
 template <int CP>
 cudaError_t pack_gt_t(const hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream_t s) {
-  if (p->tc_mode == 0) return pack_gt_cp<CP, float>(p, b0, nb, use_w, s);
-  return p->tc_fmt == 1 ? pack_gt_cp<CP, __nv_bfloat16>(p, b0, nb, use_w, s)
-                        : pack_gt_cp<CP, __half>(p, b0, nb, use_w, s);
+  if (p->tc_mode == 0) return pack_gt_cp<CP, float, 1>(p, b0, nb, use_w, s);
+  if (p->tc_mode == 1)
+    return p->tc_fmt == 1 ? pack_gt_cp<CP, __nv_bfloat16, 1>(p, b0, nb, use_w, s)
+                          : pack_gt_cp<CP, __half, 1>(p, b0, nb, use_w, s);
+  return p->tc_fmt == 1 ? pack_gt_cp<CP, __nv_bfloat16, 2>(p, b0, nb, use_w, s)
+                        : pack_gt_cp<CP, __half, 2>(p, b0, nb, use_w, s);
 }
 template <int CP>
 cudaError_t pack_at_t(const hpx_plan_s* p, const float* alm, int b0, int nb, double mfac, cudaStream_t s) {
@@ -1354,6 +1201,7 @@ cudaError_t fill_table(hpx_plan_s* p, bool col, int m0, int nm, long long base, 
 template <bool SYN>
 cudaError_t tile_all(hpx_plan_s* p, float* out, int b0, int nb, double mfac, cudaStream_t s) {
   const bool streamed = (p->flags & HPX_PLAN_LAMBDA_STREAM) != 0;
+  if (p->gen_parts == 2) return SYN ? launch_gen_synthesis(p, s) : launch_gen_analysis(p, out, mfac, s);
   if (!p->h_tab && !streamed) {
     const TileRange r{SYN ? p->tm_stab : p->tm_tab, SYN ? p->tm_stablo : p->tm_tablo, 0, p->mmax + 1, 0};
     return tile_nn<SYN>(p, out, b0, nb, mfac, r, s);
@@ -1439,6 +1287,10 @@ static_assert(kSynChannels == 8 || kSynChannels == 16 || kSynChannels == 32, "sy
 #define HPX_TC_SYN_CHANNELS_FK 32
 #endif
 constexpr int kSynChannelsFK = HPX_TC_SYN_CHANNELS_FK;
+// Channels per CTA of the tiles that generate their lambda (streamed
+// split-product plans): up to 32, whose operand tiles leave room for the
+// lambda tiles; wider transforms run the recurrence once per 32.
+constexpr int kGenChannels = 32;
 static_assert(kSynChannelsFK == 32 || kSynChannelsFK == 64, "single-product synthesis channel group");
 
 int tc_columns(int nbatch, int cap) {
@@ -1449,12 +1301,17 @@ int tc_columns(int nbatch, int cap) {
 
 int tc_channels_per_launch(const hpx_plan_s* p, bool syn) { return (syn ? p->tc_nn_s : p->tc_nn_a) / 4; }
 
-size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mode, bool host_tables) {
+static int syn_channels(int mode, bool streamed) {
+  return mode == 1 ? kSynChannelsFK : mode == 2 && streamed ? kGenChannels : kSynChannels;
+}
+static int ana_channels(int mode, bool streamed) { return mode == 0 ? 32 : mode == 2 && streamed ? kGenChannels : kAnaChannels; }
+
+size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mode, bool host_tables, bool streamed) {
   if (mode < 0) return 0;
   const size_t es = mode ? 2 : 4, kw = mode ? 64 : 32, parts = mode == 2 ? 2 : 1;
   const size_t npair = 2 * (size_t)nside, ngroup = (npair + kw - 1) / kw, nptile = (npair + 127) / 128;
-  const size_t nna = (size_t)tc_columns(nbatch, mode ? kAnaChannels : 32),
-               nns = (size_t)tc_columns(nbatch, mode == 1 ? kSynChannelsFK : kSynChannels);
+  const size_t nna = (size_t)tc_columns(nbatch, ana_channels(mode, streamed)),
+               nns = (size_t)tc_columns(nbatch, syn_channels(mode, streamed));
   size_t chunks = 0, rows = 0;
   for (int m = 0; m <= mmax; ++m) {
     chunks += (size_t)((lmax - m) / kw + 1);
@@ -1467,6 +1324,7 @@ size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mo
              + (sizeof(int) + sizeof(long long)) * (size_t)(mmax + 1) * (nptile + ngroup) +
              sizeof(long long) * (mmax + 2) + 2 * sizeof(unsigned) * nbatch;
   const size_t col = es * chunks * nptile * 128 * kw, row = es * rows * ngroup * kw;  // upper bounds, a part
+  if (mode == 2 && streamed) return b + gen_extra_bytes_estimate(nside, mmax, nbatch, 2);  // nothing staged
   if (host_tables)  // staging buffers at the default size
     return b + 2 * parts * std::min(size_t(1) << 30, (std::max(col, row) + 127) / 128 * 128);
   b += parts * col;           // column table
@@ -1563,8 +1421,8 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
   const int kw = mode ? 64 : 32, es = mode ? 2 : 4, parts = mode == 2 ? 2 : 1;
   // synthesis channels per CTA: kSynChannelsFK for one 16-bit product
   // (accumulated over all K in tensor memory), else kSynChannels
-  const int nna = tc_columns(p->nbatch, mode ? kAnaChannels : 32),
-            nns = tc_columns(p->nbatch, mode == 1 ? kSynChannelsFK : kSynChannels);
+  const int nna = tc_columns(p->nbatch, ana_channels(mode, streamed)),
+            nns = tc_columns(p->nbatch, syn_channels(mode, streamed));
   const int rba = mode == 2 ? 2 * nna : nna, rbs = mode == 2 ? 2 * nns : nns;
   auto dalloc = [&](void** ptr, size_t bytes) -> cudaError_t {
     cudaError_t e = cudaMalloc(ptr, bytes > 0 ? bytes : 16);
@@ -1678,7 +1536,9 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
     std::copy(cbm.begin(), cbm.end(), p->blk_col);
     std::copy(rbb.begin(), rbb.end(), p->blk_row_base);
     std::copy(cbb.begin(), cbb.end(), p->blk_col_base);
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = dalloc(&p->d_stage[b], p->stage_bytes * parts);
+    if (streamed && mode == 2) e = build_gen(p, 2);  // lambda never leaves the kernels
+    const bool staged = p->gen_parts != 2;
+    for (int b = 0; b < 2 && e == cudaSuccess && staged; ++b) e = dalloc(&p->d_stage[b], p->stage_bytes * parts);
     if (e != cudaSuccess) return e;
     if (host) {
       auto halloc = [&](void** ptr, size_t bytes) -> cudaError_t {
@@ -1711,7 +1571,7 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
       if (e != cudaSuccess) return e;
     }
     const unsigned long long srows = (unsigned long long)(p->stage_bytes / 128);
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < 2 && staged; ++b) {
       char* base = static_cast<char*>(p->d_stage[b]);
       if (!encode_rows128(p->tm_stage[b], base, srows, 128, es) ||
           !encode_rows128(p->tm_stagelo[b], mode == 2 ? base + p->stage_bytes : base, srows, 128, es)) {
@@ -1750,6 +1610,61 @@ cudaError_t launch_pack_tc(hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream
     case 256: return pack_gt_t<64>(p, b0, nb, use_w, s);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// FP32 plans without tensor-core tables run their analysis on the tensor cores
+// (three BF16 parts) where its cost, which hardly depends on the channels, is
+// below the CUDA-core kernel's for plans that recompute lambda and for those
+// that read the FP32 table (the two take one path, so that their results agree
+// bit for bit).  Analysis in ms, CUDA cores / tensor cores with the pack, at
+// lmax 3 Nside - 1, recomputing: Nside 256, 16 channels 0.64 / 0.43 (8: 0.32 /
+// 0.34); Nside 512, 8 channels 2.15 / 1.76; Nside 1024, 8 channels 15.7 / 10.6;
+// Nside 2048, 4 channels 137 / 76, 1 channel 52 / 75.
+int gen_parts_of(int nside, int nbatch, int dtype, unsigned flags) {
+  if (dtype != HPX_F32 || (flags & HPX_PLAN_TENSOR_CORES)) return 0;
+  const int from = nside >= 2048 ? 4 : nside >= 512 ? 8 : nside >= 256 ? 12 : INT_MAX;
+  return nbatch >= from ? 3 : 0;
+}
+
+static int gen_columns(int nbatch) { return tc_columns(nbatch, 16); }
+
+size_t gen_extra_bytes_estimate(int nside, int mmax, int nbatch, int parts) {
+  const size_t npair = 2 * (size_t)nside, state = 160 * npair * sizeof(float4);
+  if (parts != 3) return state;
+  const size_t nn = (size_t)gen_columns(nbatch), groups = ((size_t)nbatch + nn / 4 - 1) / (nn / 4);
+  return state + 2 * (size_t)(mmax + 1) * ((npair + 63) / 64) * 3 * nn * 64 * groups;
+}
+
+cudaError_t build_gen(hpx_plan_s* p, int parts) {
+  int sms = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+  if (e != cudaSuccess) return e;
+  p->gen_ctas = sms < 160 ? sms : 160;
+  const size_t state = (size_t)p->gen_ctas * p->npair * sizeof(float4);
+  e = cudaMalloc((void**)&p->d_gen_state, state);
+  if (e != cudaSuccess) return e;
+  p->bytes += state;
+  if (parts == 3) {
+    const int nn = gen_columns(p->nbatch), rows = 3 * nn;
+    p->gt_group_elems = (long long)(p->mmax + 1) * p->ngrid * rows * 64;
+    p->gt_groups = (p->nbatch + nn / 4 - 1) / (nn / 4);
+    const size_t bytes = 2 * (size_t)p->gt_group_elems * p->gt_groups;
+    e = cudaMalloc(&p->d_gt, bytes);
+    if (e != cudaSuccess) return e;
+    p->bytes += bytes;
+    if (!encode_rows128(p->tm_gt, p->d_gt, (unsigned long long)(p->gt_group_elems / 64) * p->gt_groups, nn, 2)) {
+      set_error("cuTensorMapEncodeTiled failed or is unavailable");
+      return cudaErrorInvalidValue;
+    }
+    p->gen_nn = nn;
+  }
+  p->gen_parts = parts;
+  return cudaSuccess;
+}
+
+cudaError_t launch_pack_gen(hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream_t s) {
+  return p->gen_nn == 64 ? pack_gt_cp<16, __nv_bfloat16, 3>(p, b0, nb, use_w, s)
+                         : pack_gt_cp<8, __nv_bfloat16, 3>(p, b0, nb, use_w, s);
 }
 
 cudaError_t launch_tile_tc(hpx_plan_s* p, float* alm, int b0, int nb, double mfac, cudaStream_t s) {

@@ -220,8 +220,8 @@ class GpuExecutor:
 
     table_nsides: geometries whose slots hold a plan-time lambda table on the
     tensor cores (FP16 hi/lo split products, FP32 accuracy); streamed_nsides:
-    geometries whose slots recompute lambda per call into streamed blocks
-    contracted on the tensor cores (no table held; one recurrence per
+    geometries whose slots recompute lambda per call beside the products on
+    the tensor cores (no table held; one recurrence per
     batch whatever its channel count); the others recompute lambda on the
     CUDA cores, once per group of channels of a launch.
     batch_channels: channels per batch by Nside (default 32); one batch runs

@@ -1,4 +1,9 @@
-// Ring Fourier stage of the HEALPix SHT (Sec. III-D Eq. 13, Sec. III-E).
+// Ring Fourier stage of the HEALPix SHT (Sec. III-D Eq. 13, Sec. III-E): FP64
+// plans, and the analysis of the 16-bit single-product plans in FP32.  Those
+// round the spectrum to 16 bits, which makes a last-bit difference of it one of
+// 2^-9 in some operands: the FP32 plans' transform (hpx_fft_f32.cu, a quarter
+// faster) moved their coefficients by 2.5e-5 (relative L2; 5e-3 at most) at an
+// unchanged error of 3e-3, so they keep this one and their results.
 //
 // Every ring y holds N_y = 4i (polar caps) or 4 nside (equatorial belt)
 // equally spaced pixels.  A real ring of length N is transformed through a
@@ -644,10 +649,9 @@ __global__ void k_build_bluestein(const RingInfo* __restrict__ rings, const doub
 }
 
 template <typename T>
-cudaError_t build_fft_tables(hpx_plan_s* p, cudaStream_t s) {
+static cudaError_t build_tables(hpx_plan_s* p, cudaStream_t s) {
   using V = C2<T>;
   const int ns = p->nside;
-  k_build_etab<T><<<dim3(32, ns), 256, 0, s>>>(ns, (V*)p->d_etab);
   if (ns > 1) k_build_chirp<T><<<dim3(8, ns - 1), 256, 0, s>>>(ns, (V*)p->d_chirp);
   k_build_twiddles<T><<<32, 256, 0, s>>>(p->logtw, (V*)p->d_tw);
   cudaError_t e = cudaGetLastError();
@@ -666,6 +670,26 @@ cudaError_t build_fft_tables(hpx_plan_s* p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   return e;
+}
+
+template <> cudaError_t build_fft_tables<double>(hpx_plan_s* p, cudaStream_t s) {
+  k_build_etab<double><<<dim3(32, p->nside), 256, 0, s>>>(p->nside, (double2*)p->d_etab);
+  return build_tables<double>(p, s);
+}
+// The FP32 plan with this file's tables (etab is the same).
+static hpx_plan_s view16(const hpx_plan_s* p) {
+  hpx_plan_s v = *p;
+  v.d_ring = p->d_ring16;
+  v.d_btab = p->d_btab16;
+  v.d_chirp = p->d_chirp16;
+  v.d_tw = p->d_tw16;
+  v.nbtab = p->nbtab16;
+  v.logm_max = v.logtw = p->logm16;
+  return v;
+}
+cudaError_t build_fft_tables16(hpx_plan_s* p, cudaStream_t s) {
+  hpx_plan_s v = view16(p);
+  return build_tables<float>(&v, s);
 }
 
 // Launch shapes.  The belt rings (2 nside + 1 of them, H = 2 nside) are one
@@ -696,18 +720,12 @@ static int cap_logm(int i) {  // log2 of the transform length of cap ring i (as 
   while ((1LL << L) < M) ++L;
   return L;
 }
-// Below this Nside the transforms are small enough to be bound by launch
-// latency (Nside 32: 131 us for an FP64 analysis + synthesis as two launches
-// a stage on one stream, 197 us as four on two), and every cap ring fits 64
-// threads anyway: one cap launch, no second stream.
-constexpr int kSplitNside = 512;
-
 static int ring_launches(const hpx_plan_s* p, RingLaunch* out) {
   const int ns = p->nside;
   int logh = 0;
   while ((1 << logh) < 2 * ns) ++logh;
   int k = 0;
-  const bool split = ns >= kSplitNside;
+  const bool split = ns >= kRingSplitNside;
   out[k++] = {0, 0, 0, 2 * ns + 1, logh, fft_threads(logh), split ? 1 : 0};
   if (ns < 2) return k;
   int lc = 0;
@@ -732,7 +750,7 @@ static int ring_launches(const hpx_plan_s* p, RingLaunch* out) {
   return k;
 }
 
-int ring_launch_count(const hpx_plan_s* p) {
+template <> int ring_launch_count<double>(const hpx_plan_s* p) {
   RingLaunch ls[4];
   return ring_launches(p, ls);
 }
@@ -741,42 +759,14 @@ static dim3 grid_of(const RingLaunch& L, int nbatch) {
   return dim3(nbatch, L.nslots);  // a ring's channels adjacent: its tables are read once from HBM
 }
 
-// The launches of the second stream run beside those on the caller's
-// stream: forked from the caller's stream before the launches and joined
-// back after them, so the call stays ordered on the caller's stream (and
-// captures into a graph as a fork and a join).  `which` picks the stream and
-// events of the analysis (0) or the synthesis (1).
-struct Fork {
-  cudaStream_t s, side;
-  cudaEvent_t join_ev = nullptr;
-  Fork(const hpx_plan_s* p, int which, cudaStream_t s_, cudaError_t& e) : s(s_), side(s_) {
-    if (!p->fft_streams || p->nside < kSplitNside || e != cudaSuccess) return;
-    cudaStream_t st = static_cast<cudaStream_t*>(p->fft_streams)[which];
-    cudaEvent_t* ev = static_cast<cudaEvent_t*>(p->fft_events) + 2 * which;
-    e = cudaEventRecord(ev[0], s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev[0], 0);
-    if (e == cudaSuccess) {
-      side = st;
-      join_ev = ev[1];
-    }
-  }
-  cudaError_t join(cudaError_t e) {
-    if (!join_ev) return e;
-    cudaError_t e2 = cudaEventRecord(join_ev, side);
-    if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(s, join_ev, 0);
-    return e != cudaSuccess ? e : e2;
-  }
-};
-
 template <typename T>
-cudaError_t launch_r2c(const hpx_plan_s* p, const T* map, cudaStream_t s) {
+static cudaError_t r2c(const hpx_plan_s* p, const T* map, unsigned* bmax, cudaStream_t s) {
   using V = C2<T>;
   cudaError_t e = allow_max_smem(k_ring_r2c<T>);
   // tensor-core plans with 16-bit operands record each channel's largest
   // spectrum component here (zeroed first)
-  unsigned* bmax = (sizeof(T) == 4 && p->tc_mode > 0) ? p->d_bmax : nullptr;
   if (e == cudaSuccess && bmax) e = cudaMemsetAsync(bmax, 0, sizeof(unsigned) * p->nbatch, s);
-  Fork f(p, 0, s, e);
+  RingFork f(p, 0, s, e);
   RingLaunch ls[4];
   const int nl = ring_launches(p, ls);
   for (int i = 0; i < nl; ++i) {
@@ -791,12 +781,20 @@ cudaError_t launch_r2c(const hpx_plan_s* p, const T* map, cudaStream_t s) {
   return f.join(e);
 }
 
-template <typename T>
-cudaError_t launch_c2r(const hpx_plan_s* p, T* map, bool scale_by_weight, cudaStream_t s) {
-  using V = C2<T>;
+template <> cudaError_t launch_r2c<double>(const hpx_plan_s* p, const double* map, cudaStream_t s) {
+  return r2c<double>(p, map, nullptr, s);
+}
+cudaError_t launch_r2c16(const hpx_plan_s* p, const float* map, cudaStream_t s) {
+  const hpx_plan_s v = view16(p);
+  return r2c<float>(&v, map, p->d_bmax, s);
+}
+
+template <> cudaError_t launch_c2r<double>(const hpx_plan_s* p, double* map, bool scale_by_weight, cudaStream_t s) {
+  using T = double;
+  using V = double2;
   cudaError_t e = allow_max_smem(k_ring_c2r<T, 256>);
   if (e == cudaSuccess) e = allow_max_smem(k_ring_c2r<T, 512>);
-  Fork f(p, 1, s, e);
+  RingFork f(p, 1, s, e);
   RingLaunch ls[4];
   const int nl = ring_launches(p, ls);
   for (int i = 0; i < nl; ++i) {
@@ -811,12 +809,5 @@ cudaError_t launch_c2r(const hpx_plan_s* p, T* map, bool scale_by_weight, cudaSt
   }
   return f.join(e);
 }
-
-template cudaError_t build_fft_tables<float>(hpx_plan_s*, cudaStream_t);
-template cudaError_t build_fft_tables<double>(hpx_plan_s*, cudaStream_t);
-template cudaError_t launch_r2c<float>(const hpx_plan_s*, const float*, cudaStream_t);
-template cudaError_t launch_r2c<double>(const hpx_plan_s*, const double*, cudaStream_t);
-template cudaError_t launch_c2r<float>(const hpx_plan_s*, float*, bool, cudaStream_t);
-template cudaError_t launch_c2r<double>(const hpx_plan_s*, double*, bool, cudaStream_t);
 
 }  // namespace hpx

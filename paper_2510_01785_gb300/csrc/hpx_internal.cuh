@@ -38,14 +38,32 @@ struct RingInfo {
   long long start;    // first pixel in RING order
   long long specoff;  // offset of its half spectrum (N/2 + 1 bins) in the spectrum workspace
   long long etab;     // offset of its table E_N[r] = exp(-i pi r / N), r in [0, 2N)
-  long long btab;     // offset of its Bluestein kernel spectrum (2^logm bins), -1 if N/2 is a power of two
+  long long btab;     // offset of its Bluestein kernel spectrum, -1 if it needs none (N/2, FP32: N/4 a power of two)
   int nphi;           // N_y
   int sigma;          // phi_0 = sigma pi / N_y
-  int logm;           // log2 of the FFT length used for the ring
+  int logm;           // log2 of the FFT length used for the ring (FP32: fft32_shape)
   int pad;
   double z, sinth;    // cos(theta_y), sin(theta_y)
   double w;           // quadrature weight of every pixel on the ring (4 pi / Npix)
 };
+
+// FP32 ring transforms (hpx_fft_f32.cu): a ring of 4i pixels is two complex
+// transforms of length i over M = A^2 R points; fft32_shape is 256 A + R.  i a
+// power of two >= 16: M = i; else M >= 2i - 1 (Bluestein), i > 8.  A = 4 to M =
+// 128, 8 to 512, then 16: smaller transforms spread over more threads, and R
+// stays a small factor that M can be fitted with.
+__host__ __device__ inline int fft32_shape(int i) {
+  const int len = (i & (i - 1)) == 0 ? i : 2 * i - 1, A = len <= 128 ? 4 : len <= 512 ? 8 : 16;
+  int r = (len + A * A - 1) / (A * A);
+  if (r > 8) r += r & 1;  // radices 9, 11, 13 and 15 have no kernel
+  return r + 256 * A;
+}
+__host__ __device__ inline int fft32_len(int i) { return (fft32_shape(i) >> 8) * (fft32_shape(i) >> 8) * (fft32_shape(i) & 255); }
+__host__ __device__ inline bool fft32_bluestein(int i) { return i > 8 && (i & (i - 1)) != 0; }
+// first-pass twiddles exp(-2 pi i j / M), j < M / A, of every M
+__host__ __device__ inline int fft32_tw_offset(int A, int rad) { return 136 * (A - 4) + A * rad * (rad - 1) / 2; }
+constexpr int kFft32Twiddles = 136 * (16 - 4) + 16 * 136;
+__host__ __device__ inline long long fft32_chirp_offset(int i) { return (long long)i * (i - 1) / 2; }
 
 }  // namespace hpx
 
@@ -59,9 +77,16 @@ struct hpx_plan_s {
   long long netab, nbtab;
   hpx::RingInfo* d_ring;
   void* d_etab;        // C2<T> per distinct ring length
-  void* d_btab;        // C2<T> Bluestein kernel spectra, natural order, scaled 1/M
-  void* d_chirp;       // C2<T> per cap ring i (offset i (i - 1)): exp(-pi i n^2 / H), n < H = 2i
-  void* d_tw;          // C2<T> tw[j] = exp(-2 pi i j / 2^logtw), j < 2^(logtw-1)
+  void* d_btab;        // C2<T> Bluestein kernel spectra, scaled 1/M (FP64: natural order; FP32: conjugated, hpx_fft_f32.cu)
+  void* d_chirp;       // FP64: per cap ring i (offset i (i - 1)): exp(-pi i n^2 / H), n < H = 2i; FP32: fft32_chirp_offset,
+                       // exp(-pi i n^2 / i), n < i
+  void* d_tw;          // FP64: tw[j] = exp(-2 pi i j / 2^logtw), j < 2^(logtw-1); FP32: fft32_tw_offset
+  // 16-bit single-product plans: rings and tables as an FP64 plan's (float2),
+  // for their analysis
+  hpx::RingInfo* d_ring16;
+  void *d_btab16, *d_chirp16, *d_tw16;
+  size_t nbtab16;
+  int logm16;
   double* d_cmm;       // [mmax+1] lambda_mm / sin^m(theta) (sign included)
   double* d_coef_c;    // [nalm] recurrence coefficient c_l of mu_l = c_l z mu_{l-1} - mu_{l-2}
   float2* d_coef_cf;   // [nalm] c_l as a double-FP32 pair (hi, lo): the FP32 plans' recurrence
@@ -596,7 +621,40 @@ inline LamTab<T> lam_tab(const hpx_plan_s* p) {
   return tb;
 }
 
-// launchers (defined in hpx_fft.cu / hpx_legendre.cu)
+// From this Nside the ring launches are split by size and run on two streams;
+// below it they are bound by launch latency (Nside 32: 131 us for an FP64
+// analysis + synthesis as two launches a stage on one stream, 197 us as four on
+// two).
+constexpr int kRingSplitNside = 512;
+
+// The launches of the second stream run beside those on the caller's
+// stream: forked from the caller's stream before the launches and joined
+// back after them, so the call stays ordered on the caller's stream (and
+// captures into a graph as a fork and a join).  `which` picks the stream and
+// events of the analysis (0) or the synthesis (1).
+struct RingFork {
+  cudaStream_t s, side;
+  cudaEvent_t join_ev = nullptr;
+  RingFork(const hpx_plan_s* p, int which, cudaStream_t s_, cudaError_t& e) : s(s_), side(s_) {
+    if (!p->fft_streams || p->nside < kRingSplitNside || e != cudaSuccess) return;
+    cudaStream_t st = static_cast<cudaStream_t*>(p->fft_streams)[which];
+    cudaEvent_t* ev = static_cast<cudaEvent_t*>(p->fft_events) + 2 * which;
+    e = cudaEventRecord(ev[0], s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev[0], 0);
+    if (e == cudaSuccess) {
+      side = st;
+      join_ev = ev[1];
+    }
+  }
+  cudaError_t join(cudaError_t e) {
+    if (!join_ev) return e;
+    cudaError_t e2 = cudaEventRecord(join_ev, side);
+    if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(s, join_ev, 0);
+    return e != cudaSuccess ? e : e2;
+  }
+};
+
+// launchers (FP64: hpx_fft.cu, hpx_legendre.cu; FP32: hpx_fft_f32.cu, hpx_legendre_f32.cu)
 template <typename T>
 cudaError_t launch_r2c(const hpx_plan_s* p, const T* map, cudaStream_t s);
 template <typename T>
@@ -608,7 +666,15 @@ cudaError_t launch_analysis(const hpx_plan_s* p, T* alm, bool use_weight, double
                             int* nlaunch);
 template <typename T>
 cudaError_t launch_synthesis(const hpx_plan_s* p, const T* alm, double mfac, cudaStream_t s, int* nlaunch);
-// FP64: hpx_legendre.cu; FP32: hpx_legendre_f32.cu
+template <> cudaError_t launch_r2c<double>(const hpx_plan_s*, const double*, cudaStream_t);
+template <> cudaError_t launch_r2c<float>(const hpx_plan_s*, const float*, cudaStream_t);
+cudaError_t launch_r2c16(const hpx_plan_s* p, const float* map, cudaStream_t s);  // 16-bit single-product plans
+template <> cudaError_t launch_c2r<double>(const hpx_plan_s*, double*, bool, cudaStream_t);
+template <> cudaError_t launch_c2r<float>(const hpx_plan_s*, float*, bool, cudaStream_t);
+// ring launches of a stage
+template <typename T> int ring_launch_count(const hpx_plan_s* p);
+template <> int ring_launch_count<double>(const hpx_plan_s*);
+template <> int ring_launch_count<float>(const hpx_plan_s*);
 template <> cudaError_t launch_analysis<double>(const hpx_plan_s*, double*, bool, double, cudaStream_t, int*);
 template <> cudaError_t launch_analysis<float>(const hpx_plan_s*, float*, bool, double, cudaStream_t, int*);
 template <> cudaError_t launch_synthesis<double>(const hpx_plan_s*, const double*, double, cudaStream_t, int*);
@@ -617,6 +683,9 @@ template <> cudaError_t launch_synthesis<float>(const hpx_plan_s*, const float*,
 // plan-time table builders (hpx_fft.cu, hpx_legendre.cu)
 template <typename T>
 cudaError_t build_fft_tables(hpx_plan_s* p, cudaStream_t s);
+template <> cudaError_t build_fft_tables<double>(hpx_plan_s*, cudaStream_t);
+template <> cudaError_t build_fft_tables<float>(hpx_plan_s*, cudaStream_t);
+cudaError_t build_fft_tables16(hpx_plan_s* p, cudaStream_t s);
 cudaError_t build_recurrence_tables(hpx_plan_s* p, cudaStream_t s);
 template <typename T>
 cudaError_t build_lambda_table(hpx_plan_s* p, cudaStream_t s);

@@ -47,7 +47,7 @@ __device__ __forceinline__ long long dnextpow2(long long v) {
 //   south cap: mirror of the north cap.
 // sin(theta) comes from exact integer forms of (1 - z)(1 + z).  Also records
 // each ring's offsets into the half-spectrum workspace and the FFT tables.
-__global__ void k_ring_geometry(int nside, RingInfo* rings) {
+__global__ void k_ring_geometry(int nside, int f32, RingInfo* rings) {
   const int y = blockIdx.x * blockDim.x + threadIdx.x;
   const long long ns = nside, npix = 12 * ns * ns;
   if (y >= 4 * nside - 1) return;
@@ -67,7 +67,13 @@ __global__ void k_ring_geometry(int nside, RingInfo* rings) {
                       : ii * ii - 1;
     R.etab = 4 * ii * (ii - 1);
     const long long H = 2 * ii;
-    if ((ii & (ii - 1)) == 0) {
+    if (f32) {
+      R.logm = fft32_shape((int)ii);
+      long long off = 0;
+      for (int j = 1; j < (int)ii; ++j)
+        if (fft32_bluestein(j)) off += fft32_len(j);
+      R.btab = fft32_bluestein((int)ii) ? off : -1;
+    } else if ((ii & (ii - 1)) == 0) {
       R.logm = dlog2(H);
       R.btab = -1;
     } else {
@@ -85,7 +91,7 @@ __global__ void k_ring_geometry(int nside, RingInfo* rings) {
     R.start = 2 * ns * (ns - 1) + 4 * ns * (i - ns);
     R.specoff = (ns * ns - 1) + (i - ns) * (2 * ns + 1);
     R.etab = 4 * ns * (ns - 1);
-    R.logm = dlog2(2 * ns);
+    R.logm = f32 ? fft32_shape(nside) : dlog2(2 * ns);
     R.btab = -1;
   }
   if (south) R.z = -R.z;
@@ -149,7 +155,7 @@ static void plan_free(hpx_plan_s* p) {
       if (st[i]) cudaStreamDestroy(st[i]);
     delete[] st;
   }
-  void* ptrs[] = {p->d_ring, p->d_etab, p->d_btab, p->d_chirp, p->d_tw, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->d_coef_p,
+  void* ptrs[] = {p->d_ring, p->d_etab, p->d_btab, p->d_chirp, p->d_tw, p->d_ring16, p->d_btab16, p->d_chirp16, p->d_tw16, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->d_coef_p,
                   p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_coef_pp, p->d_lgrid, p->d_gstart, p->d_zf,
                   p->d_gen_state, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
                   p->d_tab, p->d_tab_off, p->d_tab_lstart, p->d_gt, p->d_status, p->d_at, p->d_achunk,
@@ -204,14 +210,11 @@ static cudaError_t staged(hpx_plan_s* p, int stage, cudaStream_t s, F&& f) {
   return e != cudaSuccess ? e : e2;
 }
 
-// kernel launches of one ring-transform stage (hpx_fft.cu)
-int ring_launch_count(const hpx_plan_s* p);
-
 template <typename T>
 static cudaError_t run_analysis(hpx_plan_s* p, const void* map, void* alm, bool weighted, double mfac,
                                 cudaStream_t s) {
   cudaError_t e = staged(p, 0, s, [&](int* n) {
-    *n = ring_launch_count(p);  // belt and cap rings
+    *n = ring_launch_count<T>(p);  // belt and cap rings
     return launch_r2c<T>(p, static_cast<const T*>(map), s);
   });
   if (e != cudaSuccess) return e;
@@ -281,7 +284,7 @@ static cudaError_t run_synthesis(hpx_plan_s* p, const void* alm, void* map, bool
   }
   if (e == cudaSuccess)
     e = staged(p, 3, s, [&](int* n) {
-      *n = ring_launch_count(p);
+      *n = ring_launch_count<T>(p);
       return launch_c2r<T>(p, static_cast<T*>(map), weighted, s);
     });
   return e;
@@ -335,6 +338,24 @@ int64_t hpx_nalm(int lmax, int mmax) {
 }
 
 const char* hpx_last_error(void) { return g_err.c_str(); }
+
+// Elements of the Bluestein kernel spectra; *logm_max: log2 of the longest
+// FP64 ring transform.
+static size_t kernel_spectra(int nside, bool f64, int* logm_max) {
+  size_t n = 0;
+  *logm_max = ilog2(2LL * nside);
+  for (int i = 1; i < nside; ++i) {
+    if (!f64) {
+      if (fft32_bluestein(i)) n += (size_t)fft32_len(i);
+    } else if (!is_pow2(i)) {
+      long long M = 1;
+      while (M < 4LL * i - 1) M <<= 1;
+      n += (size_t)M;
+      if (ilog2(M) > *logm_max) *logm_max = ilog2(M);
+    }
+  }
+  return n;
+}
 
 static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dtype dtype, unsigned flags,
                               size_t stage_bytes, hpx_plan* out);
@@ -431,15 +452,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
   p->nalm = hpx_nalm(lmax, mmax);
   p->nspec = 6LL * nside * nside + 4LL * nside - 1;
   p->netab = 4LL * nside * (nside - 1) + 8LL * nside;
-  p->nbtab = 0;
-  p->logm_max = ilog2(2LL * nside);
-  for (long long i = 1; i < nside; ++i) {
-    if (is_pow2(i)) continue;
-    long long M = 1;
-    while (M < 4 * i - 1) M <<= 1;
-    p->nbtab += M;
-    if (ilog2(M) > p->logm_max) p->logm_max = ilog2(M);
-  }
+  p->nbtab = (long long)kernel_spectra(nside, dtype == HPX_F64, &p->logm_max);
   p->logtw = p->logm_max;
   const size_t rs = real_size(p), cs = 2 * rs;
   const long long nchain = (long long)(mmax + 1) * p->npair;
@@ -456,10 +469,15 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
     return true;
   };
   const bool f64 = dtype == HPX_F64;
+  const bool tc1 = tc_mode_of(dtype, flags) == 1;
+  if (tc1) p->nbtab16 = kernel_spectra(nside, true, &p->logm16);
   bool ok = alloc((void**)&p->d_ring, sizeof(RingInfo) * p->nring) &&
+            (!tc1 || (alloc((void**)&p->d_ring16, sizeof(RingInfo) * p->nring) && alloc(&p->d_btab16, cs * p->nbtab16) &&
+                      alloc(&p->d_chirp16, cs * (size_t)nside * (nside - 1)) &&
+                      alloc(&p->d_tw16, cs * ((size_t)1 << (p->logm16 - 1))))) &&
             alloc(&p->d_etab, cs * p->netab) && alloc(&p->d_btab, cs * p->nbtab) &&
-            alloc(&p->d_chirp, cs * (size_t)nside * (nside - 1)) &&
-            alloc(&p->d_tw, cs * ((size_t)1 << (p->logtw - 1))) &&
+            alloc(&p->d_chirp, cs * (size_t)nside * (nside - 1) / (f64 ? 1 : 2)) &&
+            alloc(&p->d_tw, cs * (f64 ? (size_t)1 << (p->logtw - 1) : (size_t)kFft32Twiddles)) &&
             alloc((void**)&p->d_cmm, sizeof(double) * (mmax + 1)) &&
             alloc((void**)&p->d_coef_c, sizeof(double) * p->nalm) &&
             alloc((void**)&p->d_coef_cf, sizeof(float2) * p->nalm) &&
@@ -502,7 +520,8 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
   }
   e = cudaMemsetAsync(p->d_status, 0, sizeof(int), s);
   if (e == cudaSuccess) {
-    k_ring_geometry<<<(p->nring + 127) / 128, 128, 0, s>>>(nside, p->d_ring);
+    k_ring_geometry<<<(p->nring + 127) / 128, 128, 0, s>>>(nside, !f64, p->d_ring);
+    if (tc1) k_ring_geometry<<<(p->nring + 127) / 128, 128, 0, s>>>(nside, 0, p->d_ring16);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = build_recurrence_tables(p, s);
@@ -514,7 +533,8 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
   if (e == cudaSuccess && (flags & HPX_PLAN_TENSOR_CORES)) e = build_tc(p, s);
   if (e == cudaSuccess)
     if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) e = build_gen(p, parts);
-  if (e == cudaSuccess) e = dtype == HPX_F64 ? build_fft_tables<double>(p, s) : build_fft_tables<float>(p, s);
+  if (e == cudaSuccess) e = f64 ? build_fft_tables<double>(p, s) : build_fft_tables<float>(p, s);
+  if (e == cudaSuccess && tc1) e = build_fft_tables16(p, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = e2;
   cudaStreamDestroy(s);
@@ -548,23 +568,22 @@ size_t hpx_plan_estimate_bytes(int nside, int lmax, int mmax, int nbatch, hpx_dt
   const size_t nalm = (size_t)hpx_nalm(lmax, mmax), nchain = (size_t)(mmax + 1) * npair;
   const size_t nspec = 6 * (size_t)nside * nside + 4 * (size_t)nside - 1;
   const size_t netab = 4 * (size_t)nside * (nside - 1) + 8 * (size_t)nside;
-  size_t nbtab = 0;
-  int logm_max = ilog2(2LL * nside);
-  for (long long i = 1; i < nside; ++i) {
-    if (is_pow2(i)) continue;
-    long long M = 1;
-    while (M < 4 * i - 1) M <<= 1;
-    nbtab += (size_t)M;
-    if (ilog2(M) > logm_max) logm_max = ilog2(M);
-  }
-  size_t b = sizeof(RingInfo) * nring + cs * netab + cs * (nbtab ? nbtab : 1) + cs * ((size_t)1 << (logm_max - 1)) +
-             cs * (size_t)nside * (nside - 1) +
+  const bool f64 = dtype == HPX_F64;
+  int logm_max = 0;
+  const size_t nbtab = kernel_spectra(nside, f64, &logm_max);
+  size_t b = sizeof(RingInfo) * nring + cs * netab + cs * (nbtab ? nbtab : 1) +
+             cs * (f64 ? (size_t)1 << (logm_max - 1) : (size_t)kFft32Twiddles) +
+             cs * (size_t)nside * (nside - 1) / (f64 ? 1 : 2) +
              sizeof(double) * (mmax + 1) + (3 * sizeof(double) + sizeof(float)) * nalm +
              (sizeof(int) + 2 * sizeof(double)) * nchain +
              (dtype == HPX_F64 ? 0 : 2 * sizeof(int) * (size_t)(mmax + 1) * ((npair + 63) / 64) + sizeof(float2) * npair) + cs * (size_t)nbatch * nspec +
              cs * (size_t)nbatch * nring * (mmax + 1);
   const size_t ngroup = (npair + 31) / 32;
   const int mode = tc_mode_of(dtype, flags);
+  if (mode == 1) {  // the analysis' own rings and tables
+    const size_t n16 = kernel_spectra(nside, true, &logm_max);
+    b += sizeof(RingInfo) * nring + cs * ((n16 ? n16 : 1) + ((size_t)1 << (logm_max - 1)) + (size_t)nside * (nside - 1));
+  }
   if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) b += gen_extra_bytes_estimate(nside, mmax, nbatch, parts);
   if (flags & (HPX_PLAN_LAMBDA_HOST | HPX_PLAN_LAMBDA_STREAM))  // no resident table; two staging buffers
     return b + sizeof(int) +

@@ -140,11 +140,11 @@ __device__ __forceinline__ long long from_xyf(int layout, long long nside, Xyf q
   return q.f * n2 + (long long)q.y * nside + q.x;  // FLAT
 }
 
-// index of pixel q in `layout`, 32-bit (Npix < 2^31)
-__device__ __forceinline__ int index_of(int layout, int nside, Xyf q) {
+// index of pixel q in layout L, 32-bit (Npix < 2^31)
+template <int L> __device__ __forceinline__ int index_of(int nside, Xyf q) {
   const int n2 = nside * nside;
-  if (layout == HPX_NESTED) return q.f * n2 + (int)(spread_bits((unsigned)q.x) | (spread_bits((unsigned)q.y) << 1));
-  if (layout == HPX_FLAT) return q.f * n2 + q.y * nside + q.x;
+  if constexpr (L == HPX_NESTED) return q.f * n2 + (int)(spread_bits((unsigned)q.x) | (spread_bits((unsigned)q.y) << 1));
+  if constexpr (L == HPX_FLAT) return q.f * n2 + q.y * nside + q.x;
   // RING: ring jr (1-based) of the face's pixel, then its position around it
   const int jr = kJr[q.f] * nside - q.x - q.y - 1;
   int nr, start, shift = 0;
@@ -165,64 +165,72 @@ __device__ __forceinline__ int index_of(int layout, int nside, Xyf q) {
   return start + jp - 1;
 }
 
-// (x, y) within a T x T tile of the i-th pixel in the target layout's order
-__device__ __forceinline__ void tile_pixel(int to, int i, int T, int logT, int& lx, int& ly) {
-  if (to == HPX_NESTED) {
+// (x, y) within a T x T tile of the i-th pixel in the order of layout TO.
+// RING: T pixels a turn c, x their number and x + y = c or c + T, so that the
+// turn is two runs of ring pixels (T in all, the diagonals' lengths being c + 1
+// and T - 1 - c).
+template <int TO> __device__ __forceinline__ void tile_pixel(int i, int T, int logT, int& lx, int& ly) {
+  if constexpr (TO == HPX_NESTED) {
     lx = (int)pack_bits((unsigned)i);
     ly = (int)pack_bits((unsigned)i >> 1);
-  } else if (to == HPX_FLAT) {
+  } else {
     lx = i & (T - 1);
     ly = i >> logT;
-  } else {
-    // diagonals c = x + y = 0 .. 2T-2 (lengths 1 .. T .. 1), x increasing
-    // along each; the second half is the first mirrored through the centre
-    const int half = T * (T + 1) / 2;
-    const bool second = i >= half;
-    const int k = second ? T * T - 1 - i : i;
-    int c = (int)((sqrtf(8.f * (float)k + 1.f) - 1.f) * 0.5f);
-    while (c * (c + 1) / 2 > k) --c;
-    while ((c + 1) * (c + 2) / 2 <= k) ++c;
-    const int pos = k - c * (c + 1) / 2;  // 0 .. c
-    if (!second) {
-      lx = pos;
-      ly = c - pos;
-    } else {
-      lx = T - 1 - pos;
-      ly = T - 1 - (c - pos);
-    }
+    if constexpr (TO == HPX_RING) ly = (ly - lx) & (T - 1);
   }
 }
 
 // out[b][index_to(q)] = in[b][index_from(q)] for every pixel q, elements of
 // E bytes.  Grid: ((nside / T)^2 tiles in Morton order, 12 faces), 256 threads.
-template <typename E>
-__global__ void __launch_bounds__(256)
-k_reorder(const E* __restrict__ in, E* __restrict__ out, int nside, int nbatch, int from, int to, int logT) {
+// Bound by index arithmetic and the latency of a pixel's loads (at many channels
+// by partial sectors of the ring runs), hidden by 64 warps a multiprocessor: the
+// layouts are template arguments, the diagonals need no square root, and the last
+// channels' loads are in flight together as the others'.  RING -> NESTED -> FLAT
+// -> RING of 5 FP32 channels at Nside 512: 111 -> 95 us (57 at the copy rate);
+// Nside 1024, 2 channels: 84 / 87 / 90 -> 62 / 51 / 54 us.  Two pixels a thread,
+// fewer warps or pairs of pixels measured slower or no faster at 5 channels, 8
+// channels x 4 pixels in flight twice as long.
+template <typename E, int FROM, int TO>
+__global__ void __launch_bounds__(256, sizeof(E) == 16 ? 6 : 8)
+k_reorder(const E* __restrict__ in, E* __restrict__ out, int nside, int nbatch, int logT) {
   const int T = 1 << logT, f = blockIdx.y;
   const int x0 = (int)pack_bits(blockIdx.x) << logT, y0 = (int)pack_bits(blockIdx.x >> 1) << logT;
   const long long npix = 12LL * nside * nside;
   for (int i = threadIdx.x; i < T * T; i += blockDim.x) {
     int lx, ly;
-    tile_pixel(to, i, T, logT, lx, ly);
+    tile_pixel<TO>(i, T, logT, lx, ly);
     const Xyf q{x0 + lx, y0 + ly, f};
-    const E* src = in + index_of(from, nside, q);
-    E* dst = out + index_of(to, nside, q);
-    int b = 0;
-    for (; b + 4 <= nbatch; b += 4) {  // four loads in flight
-      const E v0 = src[0], v1 = src[npix], v2 = src[2 * npix], v3 = src[3 * npix];
-      dst[0] = v0;
-      dst[npix] = v1;
-      dst[2 * npix] = v2;
-      dst[3 * npix] = v3;
+    const E* src = in + index_of<FROM>(nside, q);
+    E* dst = out + index_of<TO>(nside, q);
+    for (int b = 0; b < nbatch; b += 4) {
+      const int n = nbatch - b;
+      E v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c < n) v[c] = src[c * npix];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c < n) dst[c * npix] = v[c];
       src += 4 * npix;
       dst += 4 * npix;
     }
-    for (; b < nbatch; ++b) {
-      *dst = *src;
-      src += npix;
-      dst += npix;
-    }
   }
+}
+template <typename E, int FROM>
+void reorder_from(const void* in, void* out, int nside, int nbatch, int to, int logT, dim3 grid, cudaStream_t s) {
+  auto kern = to == HPX_RING     ? k_reorder<E, FROM, HPX_RING>
+              : to == HPX_NESTED ? k_reorder<E, FROM, HPX_NESTED>
+                                 : k_reorder<E, FROM, HPX_FLAT>;
+  kern<<<grid, 256, 0, s>>>((const E*)in, (E*)out, nside, nbatch, logT);
+}
+template <typename E>
+void reorder(const void* in, void* out, int nside, int nbatch, int from, int to, int logT, dim3 grid, cudaStream_t s) {
+  if (from == HPX_RING)
+    reorder_from<E, HPX_RING>(in, out, nside, nbatch, to, logT, grid, s);
+  else if (from == HPX_NESTED)
+    reorder_from<E, HPX_NESTED>(in, out, nside, nbatch, to, logT, grid, s);
+  else
+    reorder_from<E, HPX_FLAT>(in, out, nside, nbatch, to, logT, grid, s);
 }
 
 __global__ void k_layout_index(long long* __restrict__ idx, int nside, int from, int to, int* __restrict__ bad) {
@@ -286,13 +294,13 @@ hpx_status hpx_reorder(int nside, int nbatch, size_t elem_bytes, hpx_layout from
   const dim3 grid(per_side * per_side, 12);
   switch (elem_bytes) {
     case 4:
-      k_reorder<float><<<grid, 256, 0, s>>>((const float*)in, (float*)out, nside, nbatch, from, to, logT);
+      reorder<float>(in, out, nside, nbatch, from, to, logT, grid, s);
       break;
     case 8:
-      k_reorder<double><<<grid, 256, 0, s>>>((const double*)in, (double*)out, nside, nbatch, from, to, logT);
+      reorder<double>(in, out, nside, nbatch, from, to, logT, grid, s);
       break;
     case 16:
-      k_reorder<double2><<<grid, 256, 0, s>>>((const double2*)in, (double2*)out, nside, nbatch, from, to, logT);
+      reorder<double2>(in, out, nside, nbatch, from, to, logT, grid, s);
       break;
     default:
       set_error("hpx_reorder: elem_bytes must be 4, 8 or 16, got %zu", elem_bytes);

@@ -87,7 +87,7 @@ template <bool INV, typename V> __device__ __forceinline__ V rot90(V x) {
 // left unset).
 template <int R, bool INV, int NZ = R, int NO = R, typename V>
 __device__ __forceinline__ void dft_small(V (&v)[R]) {
-  static_assert((NZ == R && NO == R) || R == 16, "pruning is for radix 16");
+  static_assert(NO == R || R == 16, "outputs are pruned at radix 16");
   using T = decltype(V::x);
   if constexpr (R == 2) {
     const V a = v[0], b = v[1];
@@ -264,9 +264,40 @@ __device__ __forceinline__ void stockham_pass(V* buf, int logm, int Ns, const V*
 // `half_in`: the upper half of the input is zero (the first pass, radix 16,
 // neither reads nor transforms it); `half_out`: only the lower half of the
 // output is wanted (a last pass of radix 16 writes no other).
+// FP64 transforms of at most 512 points take radix 4 or 8 passes instead: an
+// FP64 instruction costs the same for 4 to 16 lanes of a warp as for 32, and the
+// chain of a radix-16 butterfly is the ring's time when there are few rings
+// (Nside 32, one channel: r2c 40 -> 26 us, c2r 47 -> 27 us; Nside 128, three:
+// 103 -> 81 and 120 -> 93 us).  blockDim.x >= 64.
+template <typename V> __device__ __forceinline__ bool small_radix(int logm) { return sizeof(V) == 16 && logm <= 9; }
+
+template <bool INV, typename V>
+__device__ void fft_small(V* buf, int logm, const V* __restrict__ tw, int logtw, const V* __restrict__ pre, bool half_in) {
+  const V* none = nullptr;
+  if (logm >= 8) {  // 8 8 4, 8 8 8
+    if (half_in) stockham_pass<8, 1, INV, 4>(buf, logm, 1, tw, logtw, pre);
+    else stockham_pass<8, 1, INV>(buf, logm, 1, tw, logtw, pre);
+    stockham_pass<8, 1, INV>(buf, logm, 8, tw, logtw, none);
+    if (logm == 8) stockham_pass<4, 1, INV>(buf, logm, 64, tw, logtw, none);
+    else stockham_pass<8, 1, INV>(buf, logm, 64, tw, logtw, none);
+    return;
+  }
+  int Ns = 1;
+  if (logm >= 2) {
+    if (half_in) stockham_pass<4, 1, INV, 2>(buf, logm, 1, tw, logtw, pre);
+    else stockham_pass<4, 1, INV>(buf, logm, 1, tw, logtw, pre);
+    for (Ns = 4; 4 * Ns <= 1 << logm; Ns *= 4) stockham_pass<4, 1, INV>(buf, logm, Ns, tw, logtw, none);
+  }
+  if (logm & 1) stockham_pass<2, 1, INV>(buf, logm, Ns, tw, logtw, Ns == 1 ? pre : none);
+}
+
 template <bool INV, typename V>
 __device__ void fft_pow2(V* buf, int logm, const V* __restrict__ tw, int logtw, const V* __restrict__ pre = nullptr,
                          int first = 0, bool half_in = false, bool half_out = false) {
+  if (first == 0 && small_radix<V>(logm)) {
+    fft_small<INV>(buf, logm, tw, logtw, pre, half_in);
+    return;
+  }
   int Ns = 1 << (4 * first), rest = logm - 4 * first;
   if (half_in && Ns == 1 && rest >= 4) {
     stockham_pass<16, 1, INV, 8, 16>(buf, logm, Ns, tw, logtw, pre);
@@ -312,12 +343,16 @@ __device__ __forceinline__ long long chirp_offset(int N) {
   return i * (i - 1);
 }
 
-// Ring of launch slot q: belt launches take y = nside - 1 + q; cap launches
-// take the cap rings i = ilo .. ilo + n - 1 (4i pixels) of the north cap
-// (y = i - 1), then of the south cap (y = 4 nside - 1 - i).
+// Ring of launch slot q.  Belt launches (caps = 0) take y = nside - 1 + q; cap
+// launches (1) the cap rings i = ilo .. ilo + n - 1 (4i pixels) of the north cap
+// (y = i - 1), then of the south cap (y = 4 nside - 1 - i); launches of all rings
+// (2) both caps' from the longest, then the belt's.
 __device__ __forceinline__ int slot_ring(int q, int caps, int ilo, int n, int nside) {
-  if (!caps) return nside - 1 + q;
-  return q < n ? ilo + q - 1 : 4 * nside - 1 - (ilo + q - n);
+  if (caps == 0) return nside - 1 + q;
+  if (caps == 1) return q < n ? ilo + q - 1 : 4 * nside - 1 - (ilo + q - n);
+  const int i = nside - 1 - (q >> 1);
+  if (i < 1) return nside - 1 + (q - 2 * (nside - 1));
+  return (q & 1) ? 4 * nside - 1 - i : i - 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -351,7 +386,7 @@ k_ring_r2c(const T* __restrict__ map, C2<T>* __restrict__ spec, const RingInfo* 
   // zero-padded to 2^(logm-1) (the pruned first pass reads no further)
   const V* x2 = reinterpret_cast<const V*>(map + (long long)b * npix + R.start);
   const int M = blue ? 1 << logm : H;
-  if (!blue && logm >= 4) {
+  if (!blue && logm >= 4 && !small_radix<V>(logm)) {
     // power-of-two rings: the first radix-16 pass (Ns = 1, no twiddles)
     // reads the ring straight from HBM -- butterfly j takes elements
     // j + r H/16, contiguous across the block's threads -- and writes
@@ -507,7 +542,7 @@ k_ring_c2r(const C2<T>* __restrict__ F, T* __restrict__ map, const RingInfo* __r
   // the ring is then z = IDFT_H(Z) with p[2n] = Re z[n], p[2n+1] = Im z[n].
   // Computed as conj(DFT_H(conj Z)), so conj Z (Bluestein: times the chirp,
   // zero-padded to 2^(logm-1)) is stored.
-  if (!blue && logm >= 4 && (H >> 4) <= (int)blockDim.x) {
+  if (!blue && logm >= 4 && !small_radix<V>(logm) && (H >> 4) <= (int)blockDim.x) {
     // power-of-two rings: conj Z is formed as the first radix-16 pass
     // (Ns = 1) reads its inputs j + r H/16 -- no separate pass over the
     // buffer -- and that pass writes elements 16 j + r
@@ -725,15 +760,14 @@ static int ring_launches(const hpx_plan_s* p, RingLaunch* out) {
   int logh = 0;
   while ((1 << logh) < 2 * ns) ++logh;
   int k = 0;
-  const bool split = ns >= kRingSplitNside;
-  out[k++] = {0, 0, 0, 2 * ns + 1, logh, fft_threads(logh), split ? 1 : 0};
-  if (ns < 2) return k;
   int lc = 0;
   for (int i = 1; i < ns; ++i) lc = cap_logm(i) > lc ? cap_logm(i) : lc;
-  if (!split) {  // one launch for all cap rings, everything on the caller's stream
-    out[k++] = {1, 1, ns - 1, 2 * (ns - 1), lc, fft_threads(lc), 0};
+  if (ns < kRingSplitNside) {
+    const int logm = lc > logh ? lc : logh;
+    out[k++] = {2, 0, 0, 4 * ns - 1, logm, fft_threads(logm), 0};
     return k;
   }
+  out[k++] = {0, 0, 0, 2 * ns + 1, logh, fft_threads(logh), 1};
   // i ranges (lo, hi]: (2^(lc-3), ns-1], (2^(lc-4), 2^(lc-3)], (0, 2^(lc-4)]
   int hi = ns - 1;
   for (int c = 0; c < 3 && hi >= 1; ++c) {

@@ -513,18 +513,20 @@ __device__ __forceinline__ float2 hi_of(X2 a) {
 
 constexpr int kDirect = 8;  // rings of at most 4 kDirect pixels: direct sums
 
-// A launch takes the belt (blockIdx.y = 0), or the two cap rings of every length
-// 4i, i = ihi - blockIdx.y (the longest first); blockIdx.x counts the (ring,
-// channel) of one length, so that its tables are read from HBM once.
+// A launch takes the belt (caps = 0), the two cap rings of every length 4i, i =
+// ihi - blockIdx.y (1; the longest first), or all rings, the caps' from the longest,
+// then the belt's (2).  blockIdx.x counts (ring, channel), the channels of a ring
+// side by side, so that its tables are read from HBM once.
 struct Ring32Args {
   const RingInfo* rings;
   const float2 *etab, *btab, *chirp, *tw;
   long long npix, nspec;
   int caps, ihi, nside, nb;
   __device__ __forceinline__ int ring(int r) const {
-    if (!caps) return nside - 1 + r;
-    const int i = ihi - blockIdx.y;
-    return r ? 4 * nside - 1 - i : i - 1;
+    if (caps == 0) return nside - 1 + r;
+    const int i = ihi - (caps == 1 ? (int)blockIdx.y : r >> 1);
+    if (i < 1) return nside - 1 + (r - 2 * (nside - 1));
+    return (r & 1) ? 4 * nside - 1 - i : i - 1;
   }
 };
 
@@ -924,12 +926,17 @@ int shape_threads(int i) {
 struct Launch32 {
   int caps, ilo, n, threads, side;
   size_t smem, bins;  // bins: of the synthesis's fold
-  dim3 grid(const hpx_plan_s* p) const { return dim3((caps ? 2 : 2 * p->nside + 1) * p->nbatch, n); }
+  dim3 grid(const hpx_plan_s* p) const {
+    const int rings = caps == 0 ? 2 * p->nside + 1 : caps == 1 ? 2 : 4 * p->nside - 1;
+    return dim3(rings * p->nbatch, caps == 1 ? n : 1);
+  }
 };
-// Launch shapes: the belt rings (i = nside) are one launch; from Nside 512 the
-// cap rings are three, by size (i up to nside / 2, 3/4 nside and nside - 1), each
-// with the threads and shared memory of its own longest transform, and the belt
-// launch runs on the plan's second stream beside them.
+// Launch shapes.  From Nside 512 the belt rings (i = nside) are one launch and the
+// cap rings three, by size (i up to nside / 2, 3/4 nside and nside - 1), each with
+// the threads and shared memory of its own longest transform; the belt launch
+// runs on the plan's second stream beside them.  Below, one launch of all rings
+// (two to four CTAs of any one ring would fit anyway, and the second launch's
+// latency is as long as the rings': Nside 64, 17 channels, 23 / 25 -> 19 / 20 us).
 int ring_launches32(const hpx_plan_s* p, Launch32* out) {
   const int ns = p->nside;
   const bool split = ns >= kRingSplitNside;
@@ -945,19 +952,19 @@ int ring_launches32(const hpx_plan_s* p, Launch32* out) {
     }
     out[k++] = L;
   };
-  add(0, ns, ns, split ? 1 : 0);
   if (split) {
+    add(0, ns, ns, 1);
     add(1, 3 * ns / 4 + 1, ns - 1, 0);
     add(1, ns / 2 + 1, 3 * ns / 4, 0);
     add(1, 1, ns / 2, 0);
   } else {
-    add(1, 1, ns - 1, 0);
+    add(2, 1, ns, 0);
   }
   return k;
 }
 Ring32Args ring_args(const hpx_plan_s* p, const Launch32& L) {
   return {p->d_ring, (const float2*)p->d_etab, (const float2*)p->d_btab, (const float2*)p->d_chirp, (const float2*)p->d_tw,
-          p->npix, p->nspec, L.caps, L.ilo + L.n - 1, p->nside, p->nbatch};
+          p->npix, p->nspec, L.caps, L.caps == 2 ? p->nside - 1 : L.ilo + L.n - 1, p->nside, p->nbatch};
 }
 
 }  // namespace

@@ -622,9 +622,9 @@ inline LamTab<T> lam_tab(const hpx_plan_s* p) {
 }
 
 // From this Nside the ring launches are split by size and run on two streams;
-// below it they are bound by launch latency (Nside 32: 131 us for an FP64
-// analysis + synthesis as two launches a stage on one stream, 197 us as four on
-// two).
+// below it they are bound by launch latency, and all rings are one launch (an FP64
+// analysis + synthesis at Nside 32: 96 us with the belt and the caps apart, 78 us
+// together).
 constexpr int kRingSplitNside = 512;
 
 // The launches of the second stream run beside those on the caller's

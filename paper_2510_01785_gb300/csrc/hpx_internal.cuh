@@ -695,8 +695,8 @@ cudaError_t build_lambda_table(hpx_plan_s* p, cudaStream_t s);
 // channels from b0, an operand pack and then the tile kernel.  The analysis
 // pack reads the ring spectra and the tile kernel writes alm; the synthesis
 // pack reads alm and the tile kernel writes the ring workspace d_F.  Both
-// stages pack every channel group of the transform (launch_pack_tc /
-// launch_pack_at_tc per group, into the group's Gt / At region) and then run
+// stages pack every channel group of the transform (launch_pack_tc per group,
+// launch_pack_at_tc all, into the groups' Gt / At regions) and then run
 // one tile launch over all of them (launch_tile_tc / launch_synthesis_tc with
 // nb up to the plan's nbatch).
 // The 16-bit dtypes (HPX_F32_BF16 ...) have only this path; their tables
@@ -708,7 +708,7 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s);
 int tc_channels_per_launch(const hpx_plan_s* p, bool synthesis);
 cudaError_t launch_pack_tc(hpx_plan_s* p, int b0, int nb, bool use_weight, cudaStream_t s);
 cudaError_t launch_tile_tc(hpx_plan_s* p, float* alm, int b0, int nb, double mfac, cudaStream_t s);
-cudaError_t launch_pack_at_tc(hpx_plan_s* p, const float* alm, int b0, int nb, double mfac, cudaStream_t s);
+cudaError_t launch_pack_at_tc(hpx_plan_s* p, const float* alm, double mfac, cudaStream_t s);
 cudaError_t launch_synthesis_tc(hpx_plan_s* p, int b0, int nb, cudaStream_t s);
 // lambda generated in the kernel (hpx_gen.cu): the analysis reads the packed
 // operand Gt (launch_pack_tc; launch_pack_gen for the FP32 plans, whose operand

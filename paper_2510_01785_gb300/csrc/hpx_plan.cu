@@ -266,14 +266,10 @@ static cudaError_t run_synthesis(hpx_plan_s* p, const void* alm, void* map, bool
     // tensor cores: the operand pack of every channel group (stage 5), then
     // one tile launch over all groups (stage 2), whose groups share each
     // lambda block through L2
-    const int cp = tc_channels_per_launch(p, true);
-    for (int b0 = 0; b0 < p->nbatch && e == cudaSuccess; b0 += cp) {
-      const int nb = p->nbatch - b0 < cp ? p->nbatch - b0 : cp;
-      e = staged(p, 5, s, [&](int* n) {
-        *n = p->tc_mode ? 2 : 1;  // 16-bit operands: channel maxima, then the pack
-        return launch_pack_at_tc(p, static_cast<const float*>(alm), b0, nb, mfac, s);
-      });
-    }
+    e = staged(p, 5, s, [&](int* n) {
+      *n = p->tc_mode ? 2 : 1;  // 16-bit operands: channel maxima, then the pack
+      return launch_pack_at_tc(p, static_cast<const float*>(alm), mfac, s);
+    });
     if (e == cudaSuccess)
       e = staged(p, 2, s, [&](int* n) {
         *n = 1;

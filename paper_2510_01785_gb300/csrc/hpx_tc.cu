@@ -45,11 +45,10 @@
 namespace hpx {
 namespace {
 
-// Largest |component| of each channel b0 .. b0+nb-1 of x ([b][stride]
-// complex values, n per channel), as float bits, into bmax[b] (atomic max;
-// zeroed first).
-__global__ void k_absmax(const float2* __restrict__ x, long long n, long long stride, int b0, unsigned* bmax) {
-  const int b = b0 + blockIdx.y;
+// Largest |component| of each channel of x ([b][stride] complex values, n per
+// channel), as float bits, into bmax[b] (atomic max; zeroed first).
+__global__ void k_absmax(const float2* __restrict__ x, long long n, long long stride, unsigned* bmax) {
+  const int b = blockIdx.y;
   const float2* xb = x + (long long)b * stride;
   float v = 0.f;
   const long long step = (long long)gridDim.x * blockDim.x;
@@ -184,14 +183,15 @@ k_pack_gt(const float2* __restrict__ spec, const float2* __restrict__ etab, cons
 template <int CP, typename E>
 __global__ void __launch_bounds__(128)
 k_pack_at(const float2* __restrict__ alm, const float* __restrict__ coef_pf, const long long* __restrict__ achunk,
-          E* __restrict__ at, int lmax, int mmax, long long nalm, int b0, int nb, float mfac, int x3,
+          E* __restrict__ at, long long group_elems, int lmax, int mmax, long long nalm, int nbatch, float mfac, int x3,
           const unsigned* __restrict__ bmax, float sfac) {
   constexpr int KW = Elt<E>::kw, C2N = 2 * CP, NN = 2 * C2N;
+  const int b0 = CP * blockIdx.z, nb = min(CP, nbatch - b0);  // the channel group
   const int rb = x3 ? 2 * NN : NN;
   const int m = blockIdx.y, j = blockIdx.x * (128 / KW) + threadIdx.x / KW, lane = threadIdx.x % KW;
   if (m > mmax || j > (lmax - m) / KW) return;
   const int l = m + KW * j + lane;
-  E* out = at + (achunk[m] + j) * rb * KW + lane;
+  E* out = at + blockIdx.z * group_elems + (achunk[m] + j) * rb * KW + lane;
   const bool in = l <= lmax;
   const bool odd = ((l - m) & 1) != 0;
   const long long base = alm_base(lmax, m);
@@ -1115,14 +1115,15 @@ cudaError_t pack_gt_cp(const hpx_plan_s* p, int b0, int nb, bool use_w, cudaStre
   return cudaGetLastError();
 }
 
+// every channel group in one launch (Nside 64, 17 channels in groups of 16: the
+// operands in 30 us with two launches a group, 16 us with two in all)
 template <int CP, typename E>
-cudaError_t pack_at_cp(const hpx_plan_s* p, const float* alm, int b0, int nb, double mfac, cudaStream_t s) {
+cudaError_t pack_at_cp(const hpx_plan_s* p, const float* alm, double mfac, cudaStream_t s) {
   constexpr int KW = Elt<E>::kw;
   const int nchunk0 = p->lmax / KW + 1;  // chunks of m = 0, the most
-  E* at = (E*)p->d_at + (long long)(b0 / CP) * p->at_group_elems;  // the group's region
-  k_pack_at<CP, E><<<dim3((nchunk0 + 128 / KW - 1) / (128 / KW), p->mmax + 1), 128, 0, s>>>(
-      (const float2*)alm, p->d_coef_pf, p->d_achunk, at, p->lmax, p->mmax, p->nalm, b0, nb, (float)mfac,
-      p->tc_mode == 2 ? 1 : 0, p->tc_mode ? p->d_bmax + p->bmax_stride : nullptr, p->tc_sfac_s);
+  k_pack_at<CP, E><<<dim3((nchunk0 + 128 / KW - 1) / (128 / KW), p->mmax + 1, (p->nbatch + CP - 1) / CP), 128, 0, s>>>(
+      (const float2*)alm, p->d_coef_pf, p->d_achunk, (E*)p->d_at, p->at_group_elems, p->lmax, p->mmax, p->nalm,
+      p->nbatch, (float)mfac, p->tc_mode == 2 ? 1 : 0, p->tc_mode ? p->d_bmax + p->bmax_stride : nullptr, p->tc_sfac_s);
   return cudaGetLastError();
 }
 
@@ -1160,11 +1161,11 @@ cudaError_t pack_gt_t(const hpx_plan_s* p, int b0, int nb, bool use_w, cudaStrea
                         : pack_gt_cp<CP, __half, 2>(p, b0, nb, use_w, s);
 }
 template <int CP>
-cudaError_t pack_at_t(const hpx_plan_s* p, const float* alm, int b0, int nb, double mfac, cudaStream_t s) {
-  if (p->tc_mode == 0) return pack_at_cp<CP, float>(p, alm, b0, nb, mfac, s);
-  return p->tc_fmt == 1 ? pack_at_cp<CP, __nv_bfloat16>(p, alm, b0, nb, mfac, s)
-                        : pack_at_cp<CP, __half>(p, alm, b0, nb, mfac, s);
+cudaError_t pack_at_t(const hpx_plan_s* p, const float* alm, double mfac, cudaStream_t s) {
+  if (p->tc_mode == 0) return pack_at_cp<CP, float>(p, alm, mfac, s);
+  return p->tc_fmt == 1 ? pack_at_cp<CP, __nv_bfloat16>(p, alm, mfac, s) : pack_at_cp<CP, __half>(p, alm, mfac, s);
 }
+
 template <int CP, bool SYN>
 cudaError_t tile_t(const hpx_plan_s* p, float* out, int b0, int nb, double mfac, const TileRange& r,
                    cudaStream_t s) {
@@ -1256,13 +1257,12 @@ int tc_mode_of(int dtype, unsigned flags) {
 namespace {
 
 // (the synthesis half of the plan's maxima)
-cudaError_t absmax(hpx_plan_s const* p, const float2* x, long long n, long long stride, int b0, int nb,
-                   cudaStream_t s) {
+cudaError_t absmax(hpx_plan_s const* p, const float2* x, long long n, long long stride, cudaStream_t s) {
   unsigned* bm = p->d_bmax + p->bmax_stride;
-  cudaError_t e = cudaMemsetAsync(bm + b0, 0, sizeof(unsigned) * nb, s);
+  cudaError_t e = cudaMemsetAsync(bm, 0, sizeof(unsigned) * p->nbatch, s);
   if (e != cudaSuccess) return e;
   const long long blocks = (n + 1023) / 1024;  // about four values per thread
-  k_absmax<<<dim3((unsigned)(blocks < 1024 ? blocks : 1024), nb), 256, 0, s>>>(x, n, stride, b0, bm);
+  k_absmax<<<dim3((unsigned)(blocks < 1024 ? blocks : 1024), p->nbatch), 256, 0, s>>>(x, n, stride, bm);
   return cudaGetLastError();
 }
 
@@ -1671,17 +1671,17 @@ cudaError_t launch_tile_tc(hpx_plan_s* p, float* alm, int b0, int nb, double mfa
   return tile_all<false>(p, alm, b0, nb, mfac, s);
 }
 
-cudaError_t launch_pack_at_tc(hpx_plan_s* p, const float* alm, int b0, int nb, double mfac, cudaStream_t s) {
+cudaError_t launch_pack_at_tc(hpx_plan_s* p, const float* alm, double mfac, cudaStream_t s) {
   if (p->tc_mode) {  // channel scales from alm: |P_l mfac a| <= 1.2 max(mfac, 1) max|component|
     p->tc_sfac_s = 1.2f * (float)(mfac > 1.0 ? mfac : 1.0);
-    cudaError_t e = absmax(p, reinterpret_cast<const float2*>(alm), p->nalm, p->nalm, b0, nb, s);
+    cudaError_t e = absmax(p, reinterpret_cast<const float2*>(alm), p->nalm, p->nalm, s);
     if (e != cudaSuccess) return e;
   }
   switch (p->tc_nn_s) {
-    case 32: return pack_at_t<8>(p, alm, b0, nb, mfac, s);
-    case 64: return pack_at_t<16>(p, alm, b0, nb, mfac, s);
-    case 128: return pack_at_t<32>(p, alm, b0, nb, mfac, s);
-    case 256: return pack_at_t<64>(p, alm, b0, nb, mfac, s);
+    case 32: return pack_at_t<8>(p, alm, mfac, s);
+    case 64: return pack_at_t<16>(p, alm, mfac, s);
+    case 128: return pack_at_t<32>(p, alm, mfac, s);
+    case 256: return pack_at_t<64>(p, alm, mfac, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -28,6 +28,8 @@
 #include <climits>
 #include <vector>
 
+#include <type_traits>
+
 #include "hpx_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -190,12 +192,10 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
 // ---------------------------------------------------------------------------
 // Lane tiling of the (LB x 2CP) output block of one warp: each lane owns LPL
 // consecutive l and CPL consecutive real components.
-template <int C2N> struct LaneTile;
-template <> struct LaneTile<2> { static constexpr int CPL = 2, LPL = 1; };
-template <> struct LaneTile<4> { static constexpr int CPL = 4, LPL = 1; };
-template <> struct LaneTile<8> { static constexpr int CPL = 4, LPL = 2; };
-template <> struct LaneTile<16> { static constexpr int CPL = 4, LPL = 4; };
-template <> struct LaneTile<32> { static constexpr int CPL = 8, LPL = 4; };
+template <int C2N> struct LaneTile {  // LPL = C2N / CPL (LB = 32), both parities of l where CPL allows
+  static constexpr int LPL = C2N <= 4 ? 1 : C2N == 16 ? 4 : 2, CPL = C2N / LPL;
+};
+static_assert(LB == 32, "lane tiles");
 
 constexpr int kMuStride = LB + 16 / (int)sizeof(T);
 
@@ -566,35 +566,39 @@ static cudaError_t launch_analysis_sel(const hpx_plan_s* p, T* alm, bool use_w, 
                   : launch_analysis_cp<CP, false>(p, alm, use_w, mfac, s, nlaunch);
 }
 
+// f(integral_constant CP) for cp = 1 .. 8
+template <typename F> static auto with_cp(int cp, F f) {
+  switch (cp) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    default: return f(std::integral_constant<int, 8>{});
+  }
+}
+// Channels a launch: as many launches as eight at most a launch need, of equal
+// width.  The FP64 pipe bounds both stages, at two instructions for the
+// recurrence and two a channel, so channels that are not there cost as much as
+// those that are (Nside 128, three channels, widths 4 -> 3: analysis 0.438 -> 0.362
+// ms, synthesis 0.481 -> 0.387; Nside 512, five, 8 -> 5: 8.88 -> 6.14 and 6.75 ->
+// 4.54 ms).
+static int channels_of(int nbatch, int launches) { return (nbatch + launches - 1) / launches; }
 static int pick_cp(const hpx_plan_s* p) {
   int nthr, csize;
   analysis_shape(p->npair, &nthr, &csize);
-  const int cmax = 8;
-  int cp = 1;
-  while (cp < p->nbatch && cp < cmax) cp *= 2;
-  auto fits = [&](int c) {
-    size_t sm = 0;
-    switch (c) {
-      case 1: sm = analysis_smem<1>(nthr); break;
-      case 2: sm = analysis_smem<2>(nthr); break;
-      case 4: sm = analysis_smem<4>(nthr); break;
-      default: sm = analysis_smem<8>(nthr); break;
-    }
-    return sm <= 200 * 1024;
-  };
-  while (cp > 1 && !fits(cp)) cp /= 2;
-  return cp;
+  auto fits = [&](int c) { return with_cp(c, [&](auto k) { return analysis_smem<decltype(k)::value>(nthr); }) <= 200 * 1024; };
+  int k = (p->nbatch + 7) / 8;
+  while (channels_of(p->nbatch, k) > 1 && !fits(channels_of(p->nbatch, k))) ++k;
+  return channels_of(p->nbatch, k);
 }
 
 template <>
 cudaError_t launch_analysis<double>(const hpx_plan_s* p, double* alm, bool use_w, double mfac, cudaStream_t s,
                                     int* nlaunch) {
-  switch (pick_cp(p)) {
-    case 1: return launch_analysis_sel<1>(p, alm, use_w, mfac, s, nlaunch);
-    case 2: return launch_analysis_sel<2>(p, alm, use_w, mfac, s, nlaunch);
-    case 4: return launch_analysis_sel<4>(p, alm, use_w, mfac, s, nlaunch);
-    default: return launch_analysis_sel<8>(p, alm, use_w, mfac, s, nlaunch);
-  }
+  return with_cp(pick_cp(p), [&](auto k) { return launch_analysis_sel<decltype(k)::value>(p, alm, use_w, mfac, s, nlaunch); });
 }
 
 template <int CP, bool TAB>
@@ -625,14 +629,8 @@ static cudaError_t launch_synthesis_sel(const hpx_plan_s* p, const T* alm, doubl
 template <>
 cudaError_t launch_synthesis<double>(const hpx_plan_s* p, const double* alm, double mfac, cudaStream_t s,
                                      int* nlaunch) {
-  int cp = 1;
-  while (cp < p->nbatch && cp < 8) cp *= 2;
-  switch (cp) {
-    case 1: return launch_synthesis_sel<1>(p, alm, mfac, s, nlaunch);
-    case 2: return launch_synthesis_sel<2>(p, alm, mfac, s, nlaunch);
-    case 4: return launch_synthesis_sel<4>(p, alm, mfac, s, nlaunch);
-    default: return launch_synthesis_sel<8>(p, alm, mfac, s, nlaunch);
-  }
+  return with_cp(channels_of(p->nbatch, (p->nbatch + 7) / 8),
+                 [&](auto k) { return launch_synthesis_sel<decltype(k)::value>(p, alm, mfac, s, nlaunch); });
 }
 
 // c_l as the double-FP32 pairs of the FP32 plans' recurrence

@@ -143,15 +143,18 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, bool& 
 }
 
 template <int CT> __device__ __forceinline__ void load_vec(float (&v)[CT], const float* src) {
-  if constexpr (CT >= 4) {
+  if constexpr (CT % 4 == 0) {
 #pragma unroll
     for (int c = 0; c < CT; c += 4) {
       const float4 q = *reinterpret_cast<const float4*>(src + c);
       v[c] = q.x, v[c + 1] = q.y, v[c + 2] = q.z, v[c + 3] = q.w;
     }
   } else {
-    const float2 q = *reinterpret_cast<const float2*>(src);
-    v[0] = q.x, v[1] = q.y;
+#pragma unroll
+    for (int c = 0; c < CT; c += 2) {
+      const float2 q = *reinterpret_cast<const float2*>(src + c);
+      v[c] = q.x, v[c + 1] = q.y;
+    }
   }
 }
 template <int CT> __device__ __forceinline__ void store_vec(float* dst, const float (&v)[CT]) {
@@ -458,7 +461,8 @@ k_legendre_synthesis_f32(const float2* __restrict__ alm, float2* __restrict__ F,
   const float mf = m > 0 ? mfac : 1.f;
   // this lane's l of a block, FQ channels at a time: fetched into registers,
   // put into shared memory once the 8 steps behind the loads are done
-  constexpr int FQ = CP >= 4 ? CP / 4 : CP;
+  constexpr int FQ = CP == 6 ? 2 : CP >= 4 ? CP / 4 : CP;
+  static_assert(CP % FQ == 0 && CP / FQ <= LB / 8, "channels fetched a block ahead");
   float2 an[FQ], cn;
   auto fetch = [&](int lb, int q) {
     const int l = lb + lane;
@@ -648,13 +652,19 @@ cudaError_t launch_analysis<float>(const hpx_plan_s* p, float* alm, bool use_w, 
 template <>
 cudaError_t launch_synthesis<float>(const hpx_plan_s* p, const float* alm, double mfac, cudaStream_t s,
                                     int* nlaunch) {
-  switch (channels(p, 16)) {
-    case 1: return launch_synthesis_sel<1>(p, alm, mfac, s, nlaunch);
-    case 2: return launch_synthesis_sel<2>(p, alm, mfac, s, nlaunch);
-    case 4: return launch_synthesis_sel<4>(p, alm, mfac, s, nlaunch);
-    case 8: return launch_synthesis_sel<8>(p, alm, mfac, s, nlaunch);
-    default: return launch_synthesis_sel<16>(p, alm, mfac, s, nlaunch);
-  }
+  // as many launches as 16 channels at most need, of the narrowest width that
+  // holds an equal share: the FP32 pipe works for channels that are not there too
+  // (Nside 256, lmax 700: 3 channels 0.127 -> 0.109 ms, 6 0.186 -> 0.160, 12 from the
+  // table 0.371 -> 0.213)
+  const int k = (p->nbatch + 15) / 16, share = (p->nbatch + k - 1) / k;
+  if (share <= 1) return launch_synthesis_sel<1>(p, alm, mfac, s, nlaunch);
+  if (share <= 2) return launch_synthesis_sel<2>(p, alm, mfac, s, nlaunch);
+  if (share <= 3) return launch_synthesis_sel<3>(p, alm, mfac, s, nlaunch);
+  if (share <= 4) return launch_synthesis_sel<4>(p, alm, mfac, s, nlaunch);
+  if (share <= 6) return launch_synthesis_sel<6>(p, alm, mfac, s, nlaunch);
+  if (share <= 8) return launch_synthesis_sel<8>(p, alm, mfac, s, nlaunch);
+  if (share <= 12) return launch_synthesis_sel<12>(p, alm, mfac, s, nlaunch);
+  return launch_synthesis_sel<16>(p, alm, mfac, s, nlaunch);
 }
 
 }  // namespace hpx

@@ -449,6 +449,26 @@ struct Chain {
     else if (((l - m) & (kRegrid - 1)) == 0) regrid(g, C);
     return grid_step(g, df_mul(Df{c[l].x, c[l].y}, z), C);
   }
+  // l .. l + 7, l - m a multiple of 8 (lg and the regrids lie on such l); zeros
+  // past lmax.  On the grid the coefficients' loads and products do not wait on
+  // the chain.
+  __device__ __forceinline__ void steps8(int l, int lmax, float (&v)[8]) {
+    if (l >= lg) {
+      float2 q[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) q[u] = c[min(l + u, lmax)];
+      if (l == lg) g = grid_enter(rc.n1, rc.n2, C);
+      else if (((l - m) & (kRegrid - 1)) == 0) regrid(g, C);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const float x = grid_step(g, df_mul(Df{q[u].x, q[u].y}, z), C);
+        v[u] = l + u <= lmax ? x : 0.f;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = l + u <= lmax ? step(l + u) : 0.f;
+    }
+  }
 };
 
 __host__ __device__ inline long long alm_base(int lmax, int m) {  // index(l = 0, m); index(l, m) = alm_base + l

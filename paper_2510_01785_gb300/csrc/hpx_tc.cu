@@ -248,7 +248,9 @@ __global__ void k_rtab_groups(const int* __restrict__ lc_tab, int lmax, int npai
   rows[(long long)m * ngroup + g] = lmax + 1 - ls;
 }
 
-// Fills m = m0 + blockIdx.y; element e of the table goes to hi[e - base]
+// Fills m = m0 + blockIdx.y, 8 steps of a chain at a time (one at a time, each waiting
+// for its coefficient, a streamed BF16 pair at Nside 512 took 3.25 ms; 2.84 now);
+// element e of the table goes to hi[e - base]
 // (base > 0 when the table is built block by block through a staging buffer).
 template <typename E>
 __global__ void k_rtab_fill(const RingInfo* __restrict__ rings, const float2* __restrict__ coef_c,
@@ -266,17 +268,23 @@ __global__ void k_rtab_fill(const RingInfo* __restrict__ rings, const float2* __
   Chain ch = chain_at<chain_scale<E>()>(rings, coef_c, lc_tab, start, lgrid, ngrid, lmax, npair, m, p);
   // rows before the warp's first chain start are zero: no recurrence there
   // (a group's warps are whole, so the early return above left all lanes)
-  const int lw = min(__reduce_min_sync(0xffffffffu, ch.lc), lmax + 1);
-  int l = ls;
-  for (; l < lw; ++l) {
-    hi[o + (long long)(l - ls) * KW] = Elt<E>::from_float(0.f);
-    if (lo) lo[o + (long long)(l - ls) * KW] = Elt<E>::from_float(0.f);
-  }
-  for (; l <= lmax; ++l) {
-    E h, r;
-    split_value<E>(p < npair ? ch.step(l) : 0.f, h, r);
-    hi[o + (long long)(l - ls) * KW] = h;
-    if (lo) lo[o + (long long)(l - ls) * KW] = r;
+  const int lw = __reduce_min_sync(0xffffffffu, ch.lc);
+  for (int l = ls; l <= lmax; l += 8) {  // ls lies on m + 128 j
+    float v[8];
+    if (l + 8 <= lw || p >= npair) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = 0.f;
+    } else {
+      ch.steps8(l, lmax, v);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (l + u > lmax) break;
+      E h, r;
+      split_value<E>(v[u], h, r);
+      hi[o + (long long)(l + u - ls) * KW] = h;
+      if (lo) lo[o + (long long)(l + u - ls) * KW] = r;
+    }
   }
 }
 
@@ -318,23 +326,25 @@ __global__ void k_ctab_fill(const RingInfo* __restrict__ rings, const float2* __
   // recurrence there (a tile's warps are whole: the early returns above
   // take all 128 threads of a tile or none)
   const int lw = __reduce_min_sync(0xffffffffu, ch.lc);
-  for (int lv = ls; lv < lend; lv += V) {
-    alignas(16) E h[V];
-    alignas(16) E r[V];
-    if (lv + V <= lw) {
+  for (int lv = ls; lv < lend; lv += 8) {
+    float v[8];
+    if (lv + 8 <= lw || p >= npair) {
 #pragma unroll
-      for (int u = 0; u < V; ++u) h[u] = r[u] = Elt<E>::from_float(0.f);
+      for (int u = 0; u < 8; ++u) v[u] = 0.f;
     } else {
-#pragma unroll
-      for (int u = 0; u < V; ++u) {
-        const int l = lv + u;
-        split_value<E>((l <= lmax && p < npair) ? ch.step(l) : 0.f, h[u], r[u]);
-      }
+      ch.steps8(lv, lmax, v);
     }
     const int q = lv - ls;
     const long long at = o + (long long)(q / KW) * 128 * KW + (q % KW);
-    *reinterpret_cast<uint4*>(hi + at) = *reinterpret_cast<const uint4*>(h);
-    if (lo) *reinterpret_cast<uint4*>(lo + at) = *reinterpret_cast<const uint4*>(r);
+#pragma unroll
+    for (int w = 0; w < 8; w += V) {
+      alignas(16) E h[V];
+      alignas(16) E r[V];
+#pragma unroll
+      for (int u = 0; u < V; ++u) split_value<E>(v[w + u], h[u], r[u]);
+      *reinterpret_cast<uint4*>(hi + at + w) = *reinterpret_cast<const uint4*>(h);
+      if (lo) *reinterpret_cast<uint4*>(lo + at + w) = *reinterpret_cast<const uint4*>(r);
+    }
   }
 }
 
@@ -402,7 +412,15 @@ struct TcShape {
   static_assert(!kLoTmem || kLoCol + 64 <= kTmemCols, "remainder buffers inside the allocation");
 };
 
-constexpr int kTcThreads = 192;  // warps 0-3 split and drain, warp 4 copies, warp 5 issues products
+// Warps 0-3 split and drain, warp 4 copies, warp 5 issues products.  The
+// single-product synthesis that fills the tensor memory (one CTA per SM, so that
+// nothing else runs beside its epilogue) has four more warps for half of its
+// channels, and the channels' scales are made once (64 BF16 channels at Nside 1024,
+// lmax 2047: 4.09 -> 3.85 ms).
+template <int NN, bool SYN, int MODE> __host__ __device__ constexpr int tc_threads() {
+  using S = TcShape<NN, SYN, MODE>;
+  return SYN && S::kFullK && S::kCtas == 1 && NN >= 64 ? 320 : 192;
+}
 
 // Synthesis CTAs of the 16-bit modes take kMq consecutive m of one pair tile:
 // each finished m's outputs wait in spare tensor-memory columns, so that the
@@ -466,7 +484,7 @@ struct TcArgs {
 // warp-collective tcgen05.ld stays convergent), waits for what it started,
 // and the CTA records the timeout.
 template <int NN, bool SYN, int MODE>
-__global__ void __launch_bounds__(kTcThreads, TcShape<NN, SYN, MODE>::kCtas)
+__global__ void __launch_bounds__((tc_threads<NN, SYN, MODE>()), (TcShape<NN, SYN, MODE>::kCtas))
 k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
               const __grid_constant__ CUtensorMap tmB, const TcArgs a) {
   using S = TcShape<NN, SYN, MODE>;
@@ -511,6 +529,7 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   int* qna = rowB + 128;    // synthesis: [MQ] blocks, first lambda row, first operand row of each m
   int* qra = qna + 4;
   int* qrb = qra + 4;
+  float* sInv = reinterpret_cast<float*>(qrb + 4);  // single-product synthesis: [C2N / 2] inverse channel scales
   auto sL = [&](int s) { return tiles + (size_t)s * S::kStage; };
   auto sB = [&](int s) { return tiles + (size_t)s * S::kStage + (MODE == 2 ? 2 : 1) * S::kA; };
   auto sBlo = [&](int s) { return tiles + (size_t)s * S::kStage + (MODE == 2 ? 2 : 1) * S::kA + S::kG; };
@@ -558,6 +577,8 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     qra[lane] = ra;
     qrb[lane] = rb;
   }
+  if (FK && SYN && warp == 2)
+    for (int c = lane; c < nbl; c += 32) sInv[c] = a.lscale / chan_scale(a.bmax, b0 + c, a.sfac);  // a power of two
   if (t == 32) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
@@ -701,7 +722,7 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     // ---- split and drain (thread t owns TMEM lane t = row t of the tile)
     const int l = l0 + t;
     const bool odd = ((l - m) & 1) != 0;
-    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+    const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     float sum[NSUM];
 #pragma unroll
     for (int j = 0; j < NSUM; ++j) sum[j] = 0.f;
@@ -883,12 +904,15 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         // region j: E (columns 0 .. C2N-1) and O (C2N .. NN-1) of the CTA's
         // j-th m (zero if it had no blocks); north ring p gets E + O, its
         // mirror E - O, a ring's nq values adjacent in F
-        const int p = ptile * 128 + t;
+        const int p = ptile * 128 + (warp & 3) * 32 + lane;
         const int ys = p == a.npair - 1 ? -1 : a.nring - 1 - p;
         float2* F = reinterpret_cast<float2*>(a.out);
         const long long mstride = a.mmax + 1;
+        // warps 6-9, where there are any, take the second half of the channels
+        constexpr int NCG = C2N / 16, HALVES = tc_threads<NN, SYN, MODE>() > 192 ? 2 : 1;
+        const int cg0 = warp >= 6 ? NCG / 2 : 0;
 #pragma unroll 1
-        for (int cg = 0; cg < C2N / 16; ++cg) {  // 8 channels: 16 E and 16 O columns
+        for (int cg = cg0; cg < cg0 + NCG / HALVES; ++cg) {  // 8 channels: 16 E and 16 O columns
           uint32_t e[MQ][16], o[MQ][16];
 #pragma unroll
           for (int j = 0; j < MQ; ++j) {
@@ -900,7 +924,7 @@ k_legendre_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
           for (int cc = 0; cc < 8; ++cc) {
             const int c = 8 * cg + cc;
             if (p < a.npair && c < nbl) {
-              const float inv = a.lscale / chan_scale(a.bmax, b0 + c, a.sfac);  // a power of two
+              const float inv = sInv[c];
 #pragma unroll
               for (int side = 0; side < 2; ++side) {
                 const int y = side ? ys : p;
@@ -1145,7 +1169,7 @@ cudaError_t tile_cp(const hpx_plan_s* p, float* out, int b0, int nb, double mfac
   a.tbase = r.tbase;
   a.ncg = ncg;
   a.cg_rows = (SYN ? p->at_group_elems : p->gt_group_elems) / (MODE == 0 ? 32 : 64);
-  k_legendre_tc<NN, SYN, MODE><<<grid, kTcThreads, TcShape<NN, SYN, MODE>::kSmem, s>>>(
+  k_legendre_tc<NN, SYN, MODE><<<grid, tc_threads<NN, SYN, MODE>(), TcShape<NN, SYN, MODE>::kSmem, s>>>(
       *reinterpret_cast<const CUtensorMap*>(r.tmA), *reinterpret_cast<const CUtensorMap*>(r.tmAlo), *tmB, a);
   return cudaGetLastError();
 }

@@ -14,19 +14,18 @@
 // done as FFT -> pointwise product with the precomputed kernel spectrum ->
 // inverse FFT, and a final chirp multiply.  One CTA handles one (ring,
 // channel); the whole transform stays in shared memory, so each stage reads
-// its input from HBM once and writes its output once.  Belt rings (all of
-// length 4 nside) and cap rings are launched separately, each launch with the
-// shared memory its longest transform needs; from Nside 512 the cap rings are
-// three launches by transform length and the belt launch runs on a second
-// stream beside them (see ring_launches); a ring's channels are adjacent
+// its input from HBM once and writes its output once.  Below Nside 512 all rings
+// are one launch; from there the belt rings (all of length 4 nside) are one, on a
+// second stream, and the cap rings three by transform length, each with the
+// shared memory its longest transform needs (see ring_launches); a ring's channels are adjacent
 // CTAs, so its chirp and kernel spectrum are read from HBM once.  Bluestein's
 // convolution input is zero in its upper half and only its lower half of
 // outputs is used, so the first forward pass and the last inverse pass are
 // pruned to those halves.
 //
 // The power-of-two FFT is a Stockham (self-sorting) transform: radix-16
-// passes, then one radix-8, -4 or -2 pass if log2 M is not a multiple of 4,
-// natural order in and out.  Each pass reads its butterflies' inputs into
+// passes, then one radix-8, -4 or -2 pass if log2 M is not a multiple of 4 (FP64
+// to 512 points: fft_small), natural order in and out.  Each pass reads its butterflies' inputs into
 // registers, synchronises, and writes the outputs.  Shared-memory element i
 // lives at i + i / 16 (one unused slot after every 16): the pass reads
 // j + r M/R and writes (j - k) R + k + r Ns, with the thread index j
@@ -358,17 +357,10 @@ __device__ __forceinline__ int slot_ring(int q, int caps, int ilo, int n, int ns
 // ---------------------------------------------------------------------------
 // analysis: real ring -> half spectrum X_y[k], k = 0..N/2 (Eq. 13)
 // ---------------------------------------------------------------------------
-// Resident CTAs per SM the ring kernels are compiled for: two of 512
-// threads (64 registers a thread) in FP32, 512 threads in FP64; the synthesis
-// kernel's build for launches of at most 256 threads takes five (48
-// registers: c2r 0.86 -> 0.80 ms at Nside 1024, 8 channels; the analysis
-// kernel measured no faster there).
-template <typename T, int MAXT> constexpr int ring_min_blocks() {
-  return sizeof(T) == 8 ? 512 / MAXT : (MAXT <= 256 ? 5 : 1024 / MAXT);
-}
-
+// Resident CTAs per SM the ring kernels are compiled for: two of 512 threads (64
+// registers a thread) in FP32, 512 threads in FP64.
 template <typename T>
-__global__ void __launch_bounds__(512, (ring_min_blocks<T, 512>()))
+__global__ void __launch_bounds__(512, (sizeof(T) == 8 ? 1 : 2))
 k_ring_r2c(const T* __restrict__ map, C2<T>* __restrict__ spec, const RingInfo* __restrict__ rings,
            const C2<T>* __restrict__ etab, const C2<T>* __restrict__ btab, const C2<T>* __restrict__ chirp,
            const C2<T>* __restrict__ tw, int logtw, long long npix, long long nspec, int caps, int ilo, int ncap,
@@ -453,7 +445,7 @@ k_ring_r2c(const T* __restrict__ map, C2<T>* __restrict__ spec, const RingInfo* 
 // D[k] = sum_{m = k mod N} F_m e^{i m phi0} + sum_{m = -k mod N, m >= 1}
 // conj(F_m e^{i m phi0}) (the aliasing fold; m = 0 contributes Re F_0).
 template <typename T, int MAXT>
-__global__ void __launch_bounds__(MAXT, (ring_min_blocks<T, MAXT>()))
+__global__ void __launch_bounds__(MAXT, 512 / MAXT)
 k_ring_c2r(const C2<T>* __restrict__ F, T* __restrict__ map, const RingInfo* __restrict__ rings,
            const C2<T>* __restrict__ etab, const C2<T>* __restrict__ btab, const C2<T>* __restrict__ chirp,
            const C2<T>* __restrict__ tw, int logtw, long long npix, int nring, int mmax,
@@ -727,15 +719,14 @@ cudaError_t build_fft_tables16(hpx_plan_s* p, cudaStream_t s) {
   return build_tables<float>(&v, s);
 }
 
-// Launch shapes.  The belt rings (2 nside + 1 of them, H = 2 nside) are one
-// launch.  From Nside 512 the cap rings (H = 2i, i < nside; Bluestein length
+// Launch shapes.  Below Nside 512 all rings are one launch.  From there the belt
+// rings (2 nside + 1 of them, H = 2 nside) are one, and the cap rings (H = 2i, i < nside; Bluestein length
 // 2^L with 4i - 1 <= 2^L < 8i - 2 unless 2i is a power of two) are three, by size:
 // the rings of the longest length 2^Lc (i > 2^(Lc-3)), of half that length
 // (i > 2^(Lc-4)), and the rest, each launch with the threads and shared
 // memory of its own longest transform, so that no CTA carries idle threads
-// for a ring a quarter of the launch's size (r2c 0.465 -> 0.440 ms, c2r
-// 0.672 -> 0.663 ms at Nside 1024, 8 channels; 3.53 -> 3.29 and 4.71 ->
-// 4.38 ms at 64).  The cap launches run on the caller's stream, the belt
+// for a ring a quarter of the launch's size (FP32 r2c 0.465 -> 0.440 ms at
+// Nside 1024, 8 channels; 3.53 -> 3.29 ms at 64).  The cap launches run on the caller's stream, the belt
 // launch on the plan's second stream beside them (the smaller cap classes
 // there too measured no faster).
 struct RingLaunch {

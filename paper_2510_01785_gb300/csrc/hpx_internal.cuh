@@ -53,15 +53,12 @@ struct RingInfo {
 // 128, 8 to 512, then 16: smaller transforms spread over more threads, and R
 // stays a small factor that M can be fitted with.
 __host__ __device__ inline int fft32_shape(int i) {
-  const int len = (i & (i - 1)) == 0 ? i : 2 * i - 1, log_a = len <= 128 ? 2 : len <= 512 ? 3 : 4;
-  int r = (len + (1 << 2 * log_a) - 1) >> 2 * log_a;
+  const int len = (i & (i - 1)) == 0 ? i : 2 * i - 1, A = len <= 128 ? 4 : len <= 512 ? 8 : 16;
+  int r = (len + A * A - 1) / (A * A);
   if (r > 8) r += r & 1;  // radices 9, 11, 13 and 15 have no kernel
-  return r + (256 << log_a);
+  return r + 256 * A;
 }
-__host__ __device__ inline int fft32_len(int i) {
-  const int code = fft32_shape(i), a = code >> 8;
-  return a * a * (code & 255);
-}
+__host__ __device__ inline int fft32_len(int i) { return (fft32_shape(i) >> 8) * (fft32_shape(i) >> 8) * (fft32_shape(i) & 255); }
 __host__ __device__ inline bool fft32_bluestein(int i) { return i > 8 && (i & (i - 1)) != 0; }
 // first-pass twiddles exp(-2 pi i j / M), j < M / A, of every M
 __host__ __device__ inline int fft32_tw_offset(int A, int rad) { return 136 * (A - 4) + A * rad * (rad - 1) / 2; }

@@ -265,7 +265,7 @@ __device__ __forceinline__ float df_real(Df x) { return fabsf(x.hi) < 0x1p-22f ?
 //   s a multiple of a fixed quantum u (2^-18 in mu).  The product is split
 //   into its multiple of u, q = (p s1 + C) - C with C = 1.5 2^23 u, and the
 //   exact rest (one FMA), so s = q - s2 is exact and needs no TwoSum; f takes
-//   the rest and the first-order terms in plain FP32.  |mu| is at most 15.4
+//   the rest and the first-order terms in plain FP32.  |mu| is at most 17.9
 //   for Nside <= 2048 (m = 0 on the first rings), so |s| < 2^23 u and q, of at
 //   most twice that, stays a multiple of u / 2.  s absorbs f's whole quanta
 //   every 16 steps (regrid), so f stays within tens of u and a step adds about
@@ -273,15 +273,17 @@ __device__ __forceinline__ float df_real(Df x) { return fabsf(x.hi) < 0x1p-22f ?
 //
 // A chain changes phase at the grid start of its 64-pair group: every chain of
 // the group has started and has |mu| >= 2^-4 (it grows from there, and a step's
-// error with it), aligned up to the 32-step blocks m + 32 k.  The groups of
-// the first Npair / 32 pairs never do from Nside 512 on: so near the pole a
-// step's error grows linearly in l.  Simulated against extended precision
-// (relative L2 over l of the worst chain): 2^-24 at Nside 2048 / lmax 6143,
-// 2^-24 .. 2^-31 elsewhere, median 2^-34, where rounding the values to FP32
-// gives 2^-26.  92% of
-// the steps at Nside 2048 / lmax 6143 are grid steps, 78% at Nside 512 / lmax
-// 1024.  Every FP32 kernel and table takes the same steps (operations rounded
-// one by one, scalar or two chains packed), so their values agree bit for bit.
+// error with it), aligned up to the 32-step blocks m + 32 k.  Near the pole a
+// step's error grows linearly in l, up to 1 / sin(theta) times itself, so that
+// a ring at theta ends with about 2^-42 lmax / theta; the groups next to the pole
+// stay in the general phase (grid_never).  Simulated against extended precision
+// (relative L2 over l of the worst chain, m = 0 .. 60): at lmax = 3 Nside - 1,
+// 2^-24.2 or less for every Nside, and so at lmax 16384 (with all groups on the grid:
+// Nside 64 2^-22, 256 2^-20.2, 2048 2^-18.8).  Rounding the values to FP32 alone
+// gives 2^-25.  92% of the steps at Nside 2048 / lmax 6143 are grid steps, 78% at
+// Nside 512 / lmax 1024.  Every FP32 kernel and table takes the same steps
+// (operations rounded one by one, scalar or two chains packed), so their values
+// agree bit for bit.
 struct RecurD {
   double z = 0.0, s0 = 0.0, s1 = 0.0, n1 = 0.0, n2 = 0.0;
   __device__ __forceinline__ void start(double z_, double s0_, double s1_) {
@@ -305,8 +307,15 @@ constexpr int kGridExp = 4;     // see above
 constexpr int kGridBlock = 32;  // the grid start's alignment relative to m
 constexpr int kRegrid = 16;     // steps between regrids
 constexpr float kGridC = 48.f;  // 1.5 2^23 u for u = 2^-18 (times the scale of scaled chains)
-// groups of 64 pairs (p0: the first) that stay in the general phase
-__host__ __device__ inline bool grid_never(int p0, int npair) { return npair >= 1024 && p0 < npair / 32; }
+// Groups of 64 pairs (p0: the first) that stay in the general phase: from Nside
+// 512 those below 1/32 of the pairs (lmax / theta = 120,000 at lmax = 3 Nside - 1,
+// the most that the bound above allows; below Nside 512 no group reaches it); from
+// lmax = 3 Nside on, at every Nside, those below the same lmax / theta, the first group
+// always.
+__host__ __device__ inline bool grid_never(int p0, int npair, int lmax) {
+  if (2 * lmax >= 3 * npair) return 196608LL * p0 < (long long)(lmax + 1) * npair;
+  return npair >= 1024 && p0 < npair / 32;
+}
 // the aligned grid start of a group whose recorded one is lg
 __host__ __device__ inline int grid_start(int m, int lg) {
   return m + (lg - m + kGridBlock - 1) / kGridBlock * kGridBlock;

@@ -163,7 +163,7 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
   const Df d0 = df_of(mu2 * kDfUp), d1 = df_of(mu1 * kDfUp);
   start[ci] = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
   int lg = lmax + 1;
-  if (k <= 0 && !grid_never(p & ~63, npair)) {
+  if (k <= 0 && !grid_never(p & ~63, npair, lmax)) {
     const float zf = (float)z;
     float x1 = (float)(mu1 * 0x1p100), x2 = (float)(mu2 * 0x1p100);
     lg = l;

@@ -607,9 +607,8 @@ k_ring_r2c_f32(const float* __restrict__ map, float2* __restrict__ spec, const R
   // the channel's largest spectrum component, for the 16-bit operand scale
   // of the tensor-core analysis (blockDim is a multiple of 32)
   if (bmax) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-    if ((t & 31) == 0) atomicMax(bmax + b, __float_as_uint(amax));
+    const unsigned wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // of non-negative floats
+    if ((t & 31) == 0) atomicMax(bmax + b, wmax);
   }
 }
 
@@ -997,9 +996,9 @@ template <> cudaError_t launch_r2c<float>(const hpx_plan_s* p, const float* map,
   cudaError_t e = allow_max_smem(k_ring_r2c_f32<kBelt>);
   if (e == cudaSuccess) e = allow_max_smem(k_ring_r2c_f32<kCaps>);
   if (e == cudaSuccess) e = allow_max_smem(k_ring_r2c_f32<kBigCaps>);
-  // tensor-core plans with 16-bit operands record each channel's largest
+  // analyses with 16-bit operands or parts record each channel's largest
   // spectrum component here (zeroed first)
-  unsigned* bmax = p->tc_mode > 0 ? p->d_bmax : nullptr;
+  unsigned* bmax = p->tc_mode > 0 || p->gen_parts == 3 ? p->d_bmax : nullptr;
   if (e == cudaSuccess && bmax) e = cudaMemsetAsync(bmax, 0, sizeof(unsigned) * p->nbatch, s);
   RingFork f(p, 0, s, e);
   Launch32 ls[4];

@@ -12,8 +12,9 @@
 // parts, three products: the same values, products and sums as the table
 // tiles, so the same bits), and by the analysis of the FP32 plans without
 // tensor-core tables, in three BF16 parts and six products: 3 x 8 significant
-// bits hold a float exactly, and the products left out are below 2^-26 of a
-// term.
+// bits hold a float exactly -- each channel's spectra are scaled by a power of two
+// (chan_scale), so that the third part of a weak channel is no BF16 subnormal --
+// and the products left out are below 2^-26 of a term.
 //
 // What bounds them is the FP32 pipe that steps the chains, 12 operations a
 // value (the filled-table version moved 8 bytes a value through HBM and
@@ -253,6 +254,7 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* t0 = reinterpret_cast<int*>(tmem_slot + 2);  // [64] first tile of each group
+  float* sInv = reinterpret_cast<float*>(t0 + 64);  // [C2N / 2] inverse channel scales
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -293,6 +295,7 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
       const int gs = a.gstart[(long long)m * a.ngrid + t];
       t0[t] = gs <= a.lmax ? (gs - m) / kTcTile : INT_MAX;
     }
+    if (t >= 64 && t < 64 + nbl) sInv[t - 64] = 1.f / chan_scale(a.bmax, b0 + t - 64, a.sfac);
     __syncthreads();
     if (warp >= 4 && warp < 4 + 2 * NST) {
       // ---- generators
@@ -513,7 +516,7 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
 #pragma unroll
             for (int c = 0; c < C2N / 2; ++c)
               if (c < nbl) {
-                const float inv = 1.f / chan_scale(a.bmax, b0 + c, a.sfac);
+                const float inv = sInv[c];
                 out[(long long)c * a.nalm] = make_float2(scale * sum[2 * c] * inv, scale * sum[2 * c + 1] * inv);
               }
           } else {
@@ -521,8 +524,9 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
 #pragma unroll
             for (int c = 0; c < C2N / 2; ++c)
               if (c < nbl) {
+                const float inv = sInv[c];  // last, as above
                 const float re = sum[2 * c], im = sum[2 * c + 1];
-                out[(long long)c * a.nalm] = make_float2(fmaf(re, P.x, re * P.y), fmaf(im, P.x, im * P.y));
+                out[(long long)c * a.nalm] = make_float2(fmaf(re, P.x, re * P.y) * inv, fmaf(im, P.x, im * P.y) * inv);
               }
           }
         }
@@ -894,6 +898,8 @@ cudaError_t launch_gen_analysis(const hpx_plan_s* p, float* alm, double mfac, cu
   a.nm = p->mmax + 1;
   a.cg_rows = p->gt_group_elems / 64;
   a.withhold = p->test_withhold;
+  a.bmax = p->d_bmax;
+  a.sfac = p->tc_sfac_a;
   const int nn = p->gen_parts == 3 ? p->gen_nn : p->tc_nn_a;
   a.ncg = (p->nbatch + nn / 4 - 1) / (nn / 4);
   if (p->gen_parts == 3) {
@@ -907,8 +913,6 @@ cudaError_t launch_gen_analysis(const hpx_plan_s* p, float* alm, double mfac, cu
     return cudaErrorInvalidValue;
   }
   a.fmt = (uint32_t)p->tc_fmt;
-  a.bmax = p->d_bmax;
-  a.sfac = p->tc_sfac_a;
   a.lscale = (float)(1.0 / kLamScale);
   switch (nn) {
     case 32: return a.fmt ? analysis_launch<32, 2, false, __nv_bfloat16>(p, a, s) : analysis_launch<32, 2, false, __half>(p, a, s);

@@ -141,7 +141,8 @@ struct hpx_plan_s {
   long long* d_achunk; // [mmax+2] first At chunk of each m
   unsigned* d_bmax;    // [2][bmax_stride] 16-bit modes: largest operand component per channel, of
                        // the analysis (spectra) and of the synthesis (alm), apart so that an
-                       // analysis and a synthesis may run on the plan at the same time
+                       // analysis and a synthesis may run on the plan at the same time; FP32
+                       // plans with gen_parts 3: [nbatch], of the analysis
   int bmax_stride;     // the plan's own nbatch (views for fewer channels keep it)
   void* d_stab;        // column lambda table: blocks of 128 pairs x (32 or 64) l
   void* d_stab_lo;     // 16-bit x3: its remainders

@@ -1135,7 +1135,7 @@ cudaError_t pack_gt_cp(const hpx_plan_s* p, int b0, int nb, bool use_w, cudaStre
   const int ngroup = p->gen_parts == 3 ? p->ngrid : p->ngroup;
   k_pack_gt<E, PARTS><<<dim3(ngroup, (p->mmax + kPackM) / kPackM, CP / kPackC), 256, smem, s>>>(
       (const float2*)p->d_spec, (const float2*)p->d_etab, p->d_ring, gt, p->npair, p->nring, ngroup,
-      p->nspec, p->mmax, 4 * CP, b0, nb, use_w ? 1 : 0, p->tc_mode ? p->d_bmax : nullptr, p->tc_sfac_a);
+      p->nspec, p->mmax, 4 * CP, b0, nb, use_w ? 1 : 0, p->tc_mode || PARTS == 3 ? p->d_bmax : nullptr, p->tc_sfac_a);
   return cudaGetLastError();
 }
 
@@ -1654,9 +1654,9 @@ static int gen_columns(int nbatch) { return tc_columns(nbatch, 16); }
 
 size_t gen_extra_bytes_estimate(int nside, int mmax, int nbatch, int parts) {
   const size_t npair = 2 * (size_t)nside, state = 160 * npair * sizeof(float4);
-  if (parts != 3) return state;
+  if (parts != 3) return state;  // (the split-product plans' maxima are in tc_extra_bytes_estimate)
   const size_t nn = (size_t)gen_columns(nbatch), groups = ((size_t)nbatch + nn / 4 - 1) / (nn / 4);
-  return state + 2 * (size_t)(mmax + 1) * ((npair + 63) / 64) * 3 * nn * 64 * groups;
+  return state + sizeof(unsigned) * (size_t)nbatch + 2 * (size_t)(mmax + 1) * ((npair + 63) / 64) * 3 * nn * 64 * groups;
 }
 
 cudaError_t build_gen(hpx_plan_s* p, int parts) {
@@ -1669,6 +1669,9 @@ cudaError_t build_gen(hpx_plan_s* p, int parts) {
   if (e != cudaSuccess) return e;
   p->bytes += state;
   if (parts == 3) {
+    e = cudaMalloc((void**)&p->d_bmax, sizeof(unsigned) * p->nbatch);
+    if (e != cudaSuccess) return e;
+    p->bytes += sizeof(unsigned) * p->nbatch;
     const int nn = gen_columns(p->nbatch), rows = 3 * nn;
     p->gt_group_elems = (long long)(p->mmax + 1) * p->ngrid * rows * 64;
     p->gt_groups = (p->nbatch + nn / 4 - 1) / (nn / 4);
@@ -1687,6 +1690,7 @@ cudaError_t build_gen(hpx_plan_s* p, int parts) {
 }
 
 cudaError_t launch_pack_gen(hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream_t s) {
+  p->tc_sfac_a = 3.0f * (use_w ? (float)p->w_max : 1.0f);  // as launch_pack_tc
   return p->gen_nn == 64 ? pack_gt_cp<16, __nv_bfloat16, 3>(p, b0, nb, use_w, s)
                          : pack_gt_cp<8, __nv_bfloat16, 3>(p, b0, nb, use_w, s);
 }

@@ -97,6 +97,11 @@ struct hpx_plan_s {
   double* d_mu0;       // [mmax+1][npair] mu_{lc-1} (FP64 plans)
   double* d_mu1;       // [mmax+1][npair] mu_{lc}
   float4* d_start;     // [mmax+1][npair] both times 2^104 as double-FP32 pairs (FP32 plans)
+  // FP16 hi/lo plans of a size that hpx_map2alm_noalloc takes: the same from
+  // 2^-kSigExp32 on, for the FP32 recurrence of that call (d_lc's later starts are
+  // exact for FP16 values only)
+  int* d_lc32;
+  float4* d_start32;
   int* d_lgrid;        // [mmax+1][ngrid] first l from which every chain of a 64-pair group has |mu| >= 2^-kGridExp
                        // and is past its start (lmax + 1 if some chain never is); FP32 plans
   int ngrid;           // 64-pair groups
@@ -193,8 +198,17 @@ namespace hpx {
 // monotonically up to there), so nothing is lost: below 2^-136 for FP32 and
 // BF16 (df_real flushes 2^9 mu below 2^-126), below 2^-34 for FP16 tables
 // (2^9 |mu| < 2^-25 rounds to zero, the remainder too).  FP16 tables start
-// 6.6% fewer rows that way at Nside 1024, lmax 3071.
+// 6.6% fewer rows that way at Nside 1024, lmax 3071.  hpx_map2alm_noalloc
+// contracts FP32 values on plans with FP16 tables too, from starts of their own
+// (d_lc32).
 constexpr int kSigExp64 = 200, kSigExp32 = 136, kSigExpHalf = 34;
+
+// Ring spectra that hpx_map2alm_noalloc has room for.
+constexpr size_t kNoallocBytes = size_t(16) << 20;
+// Whether a plan has the second set of chain starts (d_lc32).
+inline bool has_starts32(int dtype, int tc_mode, int nbatch, size_t nspec) {
+  return dtype == HPX_F32 && tc_mode > 0 && sizeof(float2) * (size_t)nbatch * nspec <= kNoallocBytes;
+}
 
 // Rows (l values) per tensor-core tile of the Legendre analysis; the lambda
 // table's group starts are aligned to this grid relative to m.

@@ -103,7 +103,7 @@ __global__ void k_recurrence_coefs(int lmax, int mmax, double* coef_c, double* c
 
 // Start of every chain (m, pair): the first l at which |mu_l| >= 2^-sig,
 // with (mu_{l-1}, mu_l) there; l_c = lmax + 1 if the chain never gets there.
-// FP32 plans (lgrid given, zeroed before): also, per group of 64 pairs, the
+// FP32 plans (lgrid, where given, zeroed before): also, per group of 64 pairs, the
 // largest over its chains of the first l past l_c at which |mu_l| >=
 // 2^-kGridExp (lmax + 1 where a chain never gets there; a plain FP32
 // recurrence finds it), and in gstart (large before) the earliest l_c.
@@ -162,6 +162,7 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
   }
   const Df d0 = df_of(mu2 * kDfUp), d1 = df_of(mu1 * kDfUp);
   start[ci] = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
+  if (!lgrid) return;
   int lg = lmax + 1;
   if (k <= 0 && !grid_never(p & ~63, npair, lmax)) {
     const float zf = (float)z;
@@ -667,6 +668,10 @@ cudaError_t build_recurrence_tables(hpx_plan_s* p, cudaStream_t s) {
   k_chain_scan<<<dim3((p->npair + 127) / 128, p->mmax + 1), 128, 0, s>>>(
       p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, sig, p->d_lc, p->d_mu0, p->d_mu1, p->d_start,
       p->d_lgrid, p->d_gstart, p->ngrid);
+  if (p->d_lc32)
+    k_chain_scan<<<dim3((p->npair + 127) / 128, p->mmax + 1), 128, 0, s>>>(
+        p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, kSigExp32, p->d_lc32, nullptr, nullptr,
+        p->d_start32, nullptr, nullptr, p->ngrid);
   return cudaGetLastError();
 }
 

@@ -38,7 +38,7 @@
 
 namespace {
 
-constexpr size_t kScratchBytes = size_t(16) << 20;
+constexpr size_t kScratchBytes = hpx::kNoallocBytes;
 constexpr int kMaxDevices = 64;
 
 // The scratch array itself.  In host code its name is only a stand-in, not a
@@ -140,7 +140,11 @@ extern "C" hpx_status hpx_map2alm_noalloc(hpx_plan plan, const void* map, void* 
     hpx_plan_s view = *plan;
     view.d_spec = scratch;
     view.timing = nullptr;
-    if (plan->tc_mode > 0) view.d_tab = nullptr;  // a 16-bit tensor-core table: recompute lambda instead
+    if (plan->tc_mode > 0) {  // a 16-bit tensor-core table: recompute lambda instead, from FP32 chain starts
+      view.d_tab = nullptr;
+      view.d_lc = plan->d_lc32;
+      view.d_start = plan->d_start32;
+    }
     view.d_bmax = nullptr;                         // no operand scales: the plan's own calls own them
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     int nlaunch = 0;

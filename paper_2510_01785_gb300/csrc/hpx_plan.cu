@@ -156,7 +156,7 @@ static void plan_free(hpx_plan_s* p) {
     delete[] st;
   }
   void* ptrs[] = {p->d_ring, p->d_etab, p->d_btab, p->d_chirp, p->d_tw, p->d_ring16, p->d_btab16, p->d_chirp16, p->d_tw16, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->d_coef_p,
-                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_coef_pp, p->d_lgrid, p->d_gstart, p->d_zf,
+                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_lc32, p->d_start32, p->d_coef_pp, p->d_lgrid, p->d_gstart, p->d_zf,
                   p->d_gen_state, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
                   p->d_tab, p->d_tab_off, p->d_tab_lstart, p->d_gt, p->d_status, p->d_at, p->d_achunk,
                   p->d_stab, p->d_stab_off, p->d_stab_lstart, p->d_tab_lo, p->d_stab_lo, p->d_bmax,
@@ -466,6 +466,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
   };
   const bool f64 = dtype == HPX_F64;
   const bool tc1 = tc_mode_of(dtype, flags) == 1;
+  const bool starts32 = has_starts32(dtype, tc_mode_of(dtype, flags), nbatch, p->nspec);
   if (tc1) p->nbtab16 = kernel_spectra(nside, true, &p->logm16);
   bool ok = alloc((void**)&p->d_ring, sizeof(RingInfo) * p->nring) &&
             (!tc1 || (alloc((void**)&p->d_ring16, sizeof(RingInfo) * p->nring) && alloc(&p->d_btab16, cs * p->nbtab16) &&
@@ -486,6 +487,8 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
                        alloc((void**)&p->d_lgrid, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
                        alloc((void**)&p->d_gstart, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
                        alloc((void**)&p->d_zf, sizeof(float2) * p->npair)) &&
+            (!starts32 || (alloc((void**)&p->d_lc32, sizeof(int) * nchain) &&
+                           alloc((void**)&p->d_start32, sizeof(float4) * nchain))) &&
             alloc(&p->d_spec, cs * (size_t)nbatch * p->nspec) &&
             alloc(&p->d_F, cs * (size_t)nbatch * p->nring * (mmax + 1)) &&
             alloc((void**)&p->d_status, sizeof(int));
@@ -580,6 +583,7 @@ size_t hpx_plan_estimate_bytes(int nside, int lmax, int mmax, int nbatch, hpx_dt
     const size_t n16 = kernel_spectra(nside, true, &logm_max);
     b += sizeof(RingInfo) * nring + cs * ((n16 ? n16 : 1) + ((size_t)1 << (logm_max - 1)) + (size_t)nside * (nside - 1));
   }
+  if (has_starts32(dtype, mode, nbatch, nspec)) b += (sizeof(int) + sizeof(float4)) * nchain;
   if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) b += gen_extra_bytes_estimate(nside, mmax, nbatch, parts);
   if (flags & (HPX_PLAN_LAMBDA_HOST | HPX_PLAN_LAMBDA_STREAM))  // no resident table; two staging buffers
     return b + sizeof(int) +

@@ -391,8 +391,10 @@ hpx_status hpx_plan_device_status(hpx_plan plan);
  * issue none of their copies, so the first wait of each CTA for a copy runs
  * out after its limit (1 s), with no copy or product in flight; the CTA
  * frees its tensor memory, writes no output and records HPX_ERR_TIMEOUT,
- * which the next hpx_plan_device_status returns.  Transforms that have no
- * tile kernel (CUDA-core plans) are unaffected.  0 restores normal work. */
+ * which the next hpx_plan_device_status returns.  Likewise the FP32 analyses
+ * on the CUDA cores withhold their blocks' sums from the warps that add them
+ * up.  FP64 plans and FP32 syntheses on the CUDA cores have no such waits
+ * and are unaffected.  0 restores normal work. */
 hpx_status hpx_plan_test_withhold_copies(hpx_plan plan, int withhold);
 
 /* Pixel layouts (Sec. III-B).

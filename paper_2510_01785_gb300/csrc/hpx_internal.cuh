@@ -184,7 +184,7 @@ struct hpx_plan_s {
   void* fft_events;    // cudaEvent_t[4]: fork / join of the analysis, then of the synthesis
   void* stage_events;  // cudaEvent_t[4]: copied[2], free[2]
   int* d_status;       // device-side wait status (HPX_OK or HPX_ERR_TIMEOUT)
-  int test_withhold;   // test support: tile kernels issue no copies (hpx_plan_test_withhold_copies)
+  int test_withhold;   // test support: tile kernels issue no copies, FP32 analyses no sums (hpx_plan_test_withhold_copies)
   double w_max;        // largest ring weight (4 pi / Npix unless set)
   size_t bytes;
 };

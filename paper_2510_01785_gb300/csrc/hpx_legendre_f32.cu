@@ -74,7 +74,10 @@ __device__ __forceinline__ float2 coef_at(const float2* __restrict__ c, int l, i
 //     r's inbox (st.async, which also completes r's in[place]), one of four
 //     places; credit[place] (an arrival from every owner) frees it;
 //   output warp: adds the cluster's slices of this CTA's l and writes alm.
-// Every wait is bounded in time.  Deterministic order.
+// Every wait is bounded in time.  Deterministic order.  A sum or output warp whose
+// wait has expired stops there: it sends nothing it has no credit for and gives no
+// more credit, so that what can still be on its way to a CTA was sent before the
+// final cluster barrier; a CTA that did not take it stays until it has landed.
 //
 // Four compute warps a CTA (256 chains; eight at Nside 2048, where clusters of
 // more than eight CTAs would be needed).
@@ -142,6 +145,17 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, bool& 
   late = true;
 }
 
+// The same by a whole warp, which gives up together.
+__device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, bool& late) {
+  if (late || __all_sync(0xffffffffu, mbar_test(bar, parity))) return;
+  const unsigned long long t0 = global_ns();
+  for (unsigned i = 1; i < (1u << 31); ++i) {
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return;
+    if ((i & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > 1000000000ull)) break;
+  }
+  late = true;
+}
+
 template <int CT> __device__ __forceinline__ void load_vec(float (&v)[CT], const float* src) {
   if constexpr (CT % 4 == 0) {
 #pragma unroll
@@ -167,14 +181,17 @@ template <int CT> __device__ __forceinline__ void store_vec(float* dst, const fl
   }
 }
 
+// (Two channels without a table: 96 registers are asked for, since 64, which the
+// compiler may choose instead, spill: Nside 128 / lmax 383 60 -> 70 us, Nside 512 / lmax
+// 1024 0.63 -> 0.65 ms.)
 template <int CP, bool TAB>
-__global__ void __launch_bounds__(320)
+__global__ void __launch_bounds__(320, (CP == 2 && !TAB ? 2 : 0))
 k_legendre_analysis_f32(const float2* __restrict__ spec, float2* __restrict__ alm, const RingInfo* __restrict__ rings,
                         const float2* __restrict__ etab, const float2* __restrict__ coef_cf,
                         const float2* __restrict__ coef_pp, const int* __restrict__ lc_tab,
                         const float4* __restrict__ start, const float2* __restrict__ zf,
                         const int* __restrict__ lgrid, int ngrid, int lmax, int npair, int nring, long long nspec, long long nalm, int b0, int nb, int use_w,
-                        const LamTab<float> tb, float mfac, int* __restrict__ status) {
+                        const LamTab<float> tb, float mfac, int* __restrict__ status, int withhold) {
   using A = ATile<CP>;
   constexpr int C2N = A::C2N, CT = A::CT, KS = A::KS, MS = A::MS, PS = A::PS, NOUT = A::NOUT;
   cg::cluster_group cluster = cg::this_cluster();
@@ -360,15 +377,16 @@ k_legendre_analysis_f32(const float2* __restrict__ spec, float2* __restrict__ al
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(full + s);
+      if (lane == 0 && !withhold) mbar_arrive(full + s);
     }
   } else if (warp == nwarp) {
     // ---- sums over the warps, sent to their owners: CTA r owns l's r NOUT / csize floats of a block
     const int slice = NOUT / csize;
     for (int b = 0; b < nblk; ++b) {
       const int s = b & 1, q = b % kInbox;
-      mbar_wait(full + s, (uint32_t)(b >> 1) & 1u, late);
-      if (b >= kInbox) mbar_wait(credit + q, (uint32_t)(b / kInbox - 1) & 1u, late);
+      mbar_wait_warp(full + s, (uint32_t)(b >> 1) & 1u, late);
+      if (b >= kInbox) mbar_wait_warp(credit + q, (uint32_t)(b / kInbox - 1) & 1u, late);
+      if (late) break;
       for (int o = 4 * lane; o < NOUT; o += 128) {
         float4 u[8];
 #pragma unroll
@@ -402,7 +420,8 @@ k_legendre_analysis_f32(const float2* __restrict__ spec, float2* __restrict__ al
       const int q = b % kInbox, l = m + b * LB + crank * nl + li;
       const float2 P = cscale(coef_at(coef_pp + base, l, lmax), mf);
       if (csize > 1 && lane == 0) mbar_expect(in + q, NOUT * sizeof(float));
-      mbar_wait(in + q, (uint32_t)(b / kInbox) & 1u, late);
+      mbar_wait_warp(in + q, (uint32_t)(b / kInbox) & 1u, late);
+      if (late) break;
       const float* src = inbox + q * NOUT + li * C2N;
       float2 v[CP];
 #pragma unroll
@@ -426,6 +445,11 @@ k_legendre_analysis_f32(const float2* __restrict__ spec, float2* __restrict__ al
   }
   if (late) atomicExch(status, (int)HPX_ERR_TIMEOUT);
   cluster.sync();  // peers may still send to this CTA
+  if (late && warp == nwarp + 1) {  // slices not taken: 20 us, a store's way to another SM takes one or two
+    const unsigned long long t0 = global_ns();
+    for (unsigned i = 0; i < (1u << 20) && global_ns() - t0 < 20000ull; ++i) {
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -595,7 +619,7 @@ cudaError_t launch_analysis_cp(const hpx_plan_s* p, float* alm, bool use_w, doub
                            (const RingInfo*)p->d_ring, (const float2*)p->d_etab, (const float2*)p->d_coef_cf,
                            (const float2*)p->d_coef_pp, (const int*)p->d_lc, (const float4*)p->d_start,
                            (const float2*)p->d_zf, (const int*)p->d_lgrid, p->ngrid, p->lmax, p->npair, p->nring,
-                           p->nspec, p->nalm, b0, nb, use_w ? 1 : 0, lam_tab<float>(p), (float)mfac, p->d_status);
+                           p->nspec, p->nalm, b0, nb, use_w ? 1 : 0, lam_tab<float>(p), (float)mfac, p->d_status, p->test_withhold);
     if (e != cudaSuccess) return e;
     ++*nlaunch;
   }

@@ -254,7 +254,6 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* t0 = reinterpret_cast<int*>(tmem_slot + 2);  // [64] first tile of each group
-  float* sInv = reinterpret_cast<float*>(t0 + 64);  // [C2N / 2] inverse channel scales
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -295,7 +294,6 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
       const int gs = a.gstart[(long long)m * a.ngrid + t];
       t0[t] = gs <= a.lmax ? (gs - m) / kTcTile : INT_MAX;
     }
-    if (t >= 64 && t < 64 + nbl) sInv[t - 64] = 1.f / chan_scale(a.bmax, b0 + t - 64, a.sfac);
     __syncthreads();
     if (warp >= 4 && warp < 4 + 2 * NST) {
       // ---- generators
@@ -464,6 +462,7 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
       // ---- drain: thread t owns row t of the tile
       const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
       const long long base = alm_base(a.lmax, m);
+      const float myinv = lane < nbl ? 1.f / chan_scale(a.bmax, b0 + lane, a.sfac) : 1.f;  // of channel b0 + lane
       for (int tile = 0; tile < ntile; ++tile) {
         const int l = m + kTcTile * tile + t;
         const bool odd = (t & 1) != 0;
@@ -507,27 +506,27 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
           ++kblk;
         }
         if (!alive) break;
-        if (l <= a.lmax) {
-          float2* out = a.out + (long long)b0 * a.nalm + base + l;
-          const float mf = m > 0 ? a.mfac : 1.f;
-          if constexpr (PARTS == 2) {
-            // as the table tiles: P_l times powers of two, the channel scale last
-            const float scale = a.coef_pf[base + l] * mf * a.lscale;
+        const bool row = l <= a.lmax;
+        float2* out = a.out + (long long)b0 * a.nalm + base + l;
+        const float mf = m > 0 ? a.mfac : 1.f;
+        if constexpr (PARTS == 2) {
+          // as the table tiles: P_l times powers of two, the channel scale last
+          const float scale = row ? a.coef_pf[base + l] * mf * a.lscale : 0.f;
 #pragma unroll
-            for (int c = 0; c < C2N / 2; ++c)
-              if (c < nbl) {
-                const float inv = sInv[c];
-                out[(long long)c * a.nalm] = make_float2(scale * sum[2 * c] * inv, scale * sum[2 * c + 1] * inv);
-              }
-          } else {
-            const float2 P = cscale(a.coef_pp[base + l], mf);
+          for (int c = 0; c < C2N / 2; ++c) {
+            const float inv = __shfl_sync(0xffffffffu, myinv, c);
+            if (row && c < nbl)
+              out[(long long)c * a.nalm] = make_float2(scale * sum[2 * c] * inv, scale * sum[2 * c + 1] * inv);
+          }
+        } else {
+          const float2 P = row ? cscale(a.coef_pp[base + l], mf) : make_float2(0.f, 0.f);
 #pragma unroll
-            for (int c = 0; c < C2N / 2; ++c)
-              if (c < nbl) {
-                const float inv = sInv[c];  // last, as above
-                const float re = sum[2 * c], im = sum[2 * c + 1];
-                out[(long long)c * a.nalm] = make_float2(fmaf(re, P.x, re * P.y) * inv, fmaf(im, P.x, im * P.y) * inv);
-              }
+          for (int c = 0; c < C2N / 2; ++c) {
+            const float inv = __shfl_sync(0xffffffffu, myinv, c);
+            if (row && c < nbl) {
+              const float re = sum[2 * c], im = sum[2 * c + 1];
+              out[(long long)c * a.nalm] = make_float2(fmaf(re, P.x, re * P.y) * inv, fmaf(im, P.x, im * P.y) * inv);
+            }
           }
         }
       }

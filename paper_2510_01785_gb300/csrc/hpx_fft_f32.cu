@@ -997,9 +997,10 @@ template <> cudaError_t launch_r2c<float>(const hpx_plan_s* p, const float* map,
   if (e == cudaSuccess) e = allow_max_smem(k_ring_r2c_f32<kCaps>);
   if (e == cudaSuccess) e = allow_max_smem(k_ring_r2c_f32<kBigCaps>);
   // analyses with 16-bit operands or parts record each channel's largest
-  // spectrum component here (zeroed first)
+  // spectrum component here (zeroed first; for the parts the analysis that read the
+  // last ones has left zeros)
   unsigned* bmax = p->tc_mode > 0 || p->gen_parts == 3 ? p->d_bmax : nullptr;
-  if (e == cudaSuccess && bmax) e = cudaMemsetAsync(bmax, 0, sizeof(unsigned) * p->nbatch, s);
+  if (e == cudaSuccess && bmax && p->tc_mode > 0) e = cudaMemsetAsync(bmax, 0, sizeof(unsigned) * p->nbatch, s);
   RingFork f(p, 0, s, e);
   Launch32 ls[4];
   const int nl = ring_launches32(p, ls);

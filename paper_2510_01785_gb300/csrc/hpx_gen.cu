@@ -148,7 +148,8 @@ struct GenArgs {
   float4* state;      // [CTA][npair] chains between tiles
   const float* coef_pf;
   const float2* coef_pp;
-  const unsigned* bmax;
+  unsigned* bmax;     // the channels' largest spectrum components; three parts: left zero
+  const float* binv;  // three parts: the inverse channel scales
   float sfac, lscale, mfac;
   float2* out;  // alm [b][nalm]
   int lmax, npair;
@@ -282,6 +283,9 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
+  // three parts: the pack has read the maxima; the next ring transform finds zeros
+  if (PARTS == 3 && blockIdx.x == 0)
+    for (int b = t; b < a.nb; b += SH::kThreads) a.bmax[b] = 0u;
   unsigned kblk = 0;        // blocks so far (copies, products, drain)
   unsigned scount[NST] = {};  // products: blocks so far of each stage
   unsigned gcount = 0;      // generators: blocks so far of their stage
@@ -462,7 +466,8 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
       // ---- drain: thread t owns row t of the tile
       const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
       const long long base = alm_base(a.lmax, m);
-      const float myinv = lane < nbl ? 1.f / chan_scale(a.bmax, b0 + lane, a.sfac) : 1.f;  // of channel b0 + lane
+      float myinv = 1.f;  // two parts: the inverse scale of channel b0 + lane
+      if (PARTS == 2 && lane < nbl) myinv = 1.f / chan_scale(a.bmax, b0 + lane, a.sfac);
       for (int tile = 0; tile < ntile; ++tile) {
         const int l = m + kTcTile * tile + t;
         const bool odd = (t & 1) != 0;
@@ -519,14 +524,15 @@ k_gen_analysis(const __grid_constant__ CUtensorMap tmB, const GenArgs a) {
               out[(long long)c * a.nalm] = make_float2(scale * sum[2 * c] * inv, scale * sum[2 * c + 1] * inv);
           }
         } else {
-          const float2 P = row ? cscale(a.coef_pp[base + l], mf) : make_float2(0.f, 0.f);
+          if (row) {
+            const float2 P = cscale(a.coef_pp[base + l], mf);
 #pragma unroll
-          for (int c = 0; c < C2N / 2; ++c) {
-            const float inv = __shfl_sync(0xffffffffu, myinv, c);
-            if (row && c < nbl) {
-              const float re = sum[2 * c], im = sum[2 * c + 1];
-              out[(long long)c * a.nalm] = make_float2(fmaf(re, P.x, re * P.y) * inv, fmaf(im, P.x, im * P.y) * inv);
-            }
+            for (int c = 0; c < C2N / 2; ++c)
+              if (c < nbl) {
+                const float inv = a.binv[b0 + c];  // a power of two
+                const float re = sum[2 * c] * inv, im = sum[2 * c + 1] * inv;
+                out[(long long)c * a.nalm] = make_float2(fmaf(re, P.x, re * P.y), fmaf(im, P.x, im * P.y));
+              }
           }
         }
       }
@@ -898,6 +904,7 @@ cudaError_t launch_gen_analysis(const hpx_plan_s* p, float* alm, double mfac, cu
   a.cg_rows = p->gt_group_elems / 64;
   a.withhold = p->test_withhold;
   a.bmax = p->d_bmax;
+  a.binv = reinterpret_cast<const float*>(p->d_bmax + p->bmax_stride);
   a.sfac = p->tc_sfac_a;
   const int nn = p->gen_parts == 3 ? p->gen_nn : p->tc_nn_a;
   a.ncg = (p->nbatch + nn / 4 - 1) / (nn / 4);

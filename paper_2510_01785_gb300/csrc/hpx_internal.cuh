@@ -147,7 +147,8 @@ struct hpx_plan_s {
   unsigned* d_bmax;    // [2][bmax_stride] 16-bit modes: largest operand component per channel, of
                        // the analysis (spectra) and of the synthesis (alm), apart so that an
                        // analysis and a synthesis may run on the plan at the same time; FP32
-                       // plans with gen_parts 3: [nbatch], of the analysis
+                       // plans with gen_parts 3: [2][nbatch], the analysis' maxima (zero between
+                       // analyses) and, from its pack on, the inverse channel scales (floats)
   int bmax_stride;     // the plan's own nbatch (views for fewer channels keep it)
   void* d_stab;        // column lambda table: blocks of 128 pairs x (32 or 64) l
   void* d_stab_lo;     // 16-bit x3: its remainders
@@ -757,7 +758,7 @@ cudaError_t launch_synthesis_tc(hpx_plan_s* p, int b0, int nb, cudaStream_t s);
 // lambda generated in the kernel (hpx_gen.cu): the analysis reads the packed
 // operand Gt (launch_pack_tc; launch_pack_gen for the FP32 plans, whose operand
 // buffers build_gen makes), the synthesis At, as the table tiles do
-cudaError_t build_gen(hpx_plan_s* p, int parts);
+cudaError_t build_gen(hpx_plan_s* p, int parts, cudaStream_t s);
 size_t gen_extra_bytes_estimate(int nside, int mmax, int nbatch, int parts);
 int gen_parts_of(int nside, int nbatch, int dtype, unsigned flags);
 cudaError_t launch_pack_gen(hpx_plan_s* p, int b0, int nb, bool use_weight, cudaStream_t s);

@@ -531,7 +531,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
     e = dtype == HPX_F64 ? build_lambda_table<double>(p, s) : build_lambda_table<float>(p, s);
   if (e == cudaSuccess && (flags & HPX_PLAN_TENSOR_CORES)) e = build_tc(p, s);
   if (e == cudaSuccess)
-    if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) e = build_gen(p, parts);
+    if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) e = build_gen(p, parts, s);
   if (e == cudaSuccess) e = f64 ? build_fft_tables<double>(p, s) : build_fft_tables<float>(p, s);
   if (e == cudaSuccess && tc1) e = build_fft_tables16(p, s);
   cudaError_t e2 = cudaStreamSynchronize(s);

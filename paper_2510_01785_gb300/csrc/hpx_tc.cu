@@ -90,7 +90,7 @@ template <typename E, int PARTS>
 __global__ void __launch_bounds__(256)
 k_pack_gt(const float2* __restrict__ spec, const float2* __restrict__ etab, const RingInfo* __restrict__ rings,
           E* __restrict__ gt, int npair, int nring, int ngroup, long long nspec, int mmax, int NN, int b0, int nb,
-          int use_w, const unsigned* __restrict__ bmax, float sfac) {
+          int use_w, const unsigned* __restrict__ bmax, float sfac, float* __restrict__ binv) {
   constexpr int KW = Elt<E>::kw;
   // dynamic shared memory only (the launch may raise its limit to the
   // device maximum): kPackM slabs, then the channel scales
@@ -101,7 +101,10 @@ k_pack_gt(const float2* __restrict__ spec, const float2* __restrict__ etab, cons
   float* csc = reinterpret_cast<float*>(smem_raw + kPackM * slab);
   if (threadIdx.x < kPackC) {
     const int c = c0 + threadIdx.x;
-    csc[threadIdx.x] = c < nb ? chan_scale(bmax, b0 + c, sfac) : 0.f;
+    const float sc = c < nb ? chan_scale(bmax, b0 + c, sfac) : 0.f;
+    csc[threadIdx.x] = sc;
+    // three parts: the inverse for the drain, which then clears the maxima
+    if (PARTS == 3 && g == 0 && m0 == 0 && c < nb) binv[b0 + c] = 1.f / sc;
   }
   __syncthreads();
   const int nch = min(kPackC, nb - c0);  // channels with data; the rest are zero rows
@@ -1135,7 +1138,8 @@ cudaError_t pack_gt_cp(const hpx_plan_s* p, int b0, int nb, bool use_w, cudaStre
   const int ngroup = p->gen_parts == 3 ? p->ngrid : p->ngroup;
   k_pack_gt<E, PARTS><<<dim3(ngroup, (p->mmax + kPackM) / kPackM, CP / kPackC), 256, smem, s>>>(
       (const float2*)p->d_spec, (const float2*)p->d_etab, p->d_ring, gt, p->npair, p->nring, ngroup,
-      p->nspec, p->mmax, 4 * CP, b0, nb, use_w ? 1 : 0, p->tc_mode || PARTS == 3 ? p->d_bmax : nullptr, p->tc_sfac_a);
+      p->nspec, p->mmax, 4 * CP, b0, nb, use_w ? 1 : 0, p->tc_mode || PARTS == 3 ? p->d_bmax : nullptr, p->tc_sfac_a,
+      PARTS == 3 ? reinterpret_cast<float*>(p->d_bmax + p->bmax_stride) : nullptr);
   return cudaGetLastError();
 }
 
@@ -1560,7 +1564,7 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
     std::copy(cbm.begin(), cbm.end(), p->blk_col);
     std::copy(rbb.begin(), rbb.end(), p->blk_row_base);
     std::copy(cbb.begin(), cbb.end(), p->blk_col_base);
-    if (streamed && mode == 2) e = build_gen(p, 2);  // lambda never leaves the kernels
+    if (streamed && mode == 2) e = build_gen(p, 2, s);  // lambda never leaves the kernels
     const bool staged = p->gen_parts != 2;
     for (int b = 0; b < 2 && e == cudaSuccess && staged; ++b) e = dalloc(&p->d_stage[b], p->stage_bytes * parts);
     if (e != cudaSuccess) return e;
@@ -1656,10 +1660,10 @@ size_t gen_extra_bytes_estimate(int nside, int mmax, int nbatch, int parts) {
   const size_t npair = 2 * (size_t)nside, state = 160 * npair * sizeof(float4);
   if (parts != 3) return state;  // (the split-product plans' maxima are in tc_extra_bytes_estimate)
   const size_t nn = (size_t)gen_columns(nbatch), groups = ((size_t)nbatch + nn / 4 - 1) / (nn / 4);
-  return state + sizeof(unsigned) * (size_t)nbatch + 2 * (size_t)(mmax + 1) * ((npair + 63) / 64) * 3 * nn * 64 * groups;
+  return state + 2 * sizeof(unsigned) * (size_t)nbatch + 2 * (size_t)(mmax + 1) * ((npair + 63) / 64) * 3 * nn * 64 * groups;
 }
 
-cudaError_t build_gen(hpx_plan_s* p, int parts) {
+cudaError_t build_gen(hpx_plan_s* p, int parts, cudaStream_t s) {
   int sms = 0;
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
   if (e != cudaSuccess) return e;
@@ -1669,9 +1673,12 @@ cudaError_t build_gen(hpx_plan_s* p, int parts) {
   if (e != cudaSuccess) return e;
   p->bytes += state;
   if (parts == 3) {
-    e = cudaMalloc((void**)&p->d_bmax, sizeof(unsigned) * p->nbatch);
+    const size_t maxima = 2 * sizeof(unsigned) * (size_t)p->nbatch;
+    e = cudaMalloc((void**)&p->d_bmax, maxima);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_bmax, 0, maxima, s);
     if (e != cudaSuccess) return e;
-    p->bytes += sizeof(unsigned) * p->nbatch;
+    p->bytes += maxima;
+    p->bmax_stride = p->nbatch;
     const int nn = gen_columns(p->nbatch), rows = 3 * nn;
     p->gt_group_elems = (long long)(p->mmax + 1) * p->ngrid * rows * 64;
     p->gt_groups = (p->nbatch + nn / 4 - 1) / (nn / 4);

@@ -999,7 +999,7 @@ template <> cudaError_t launch_r2c<float>(const hpx_plan_s* p, const float* map,
   // analyses with 16-bit operands or parts record each channel's largest
   // spectrum component here (zeroed first; for the parts the analysis that read the
   // last ones has left zeros)
-  unsigned* bmax = p->tc_mode > 0 || p->gen_parts == 3 ? p->d_bmax : nullptr;
+  unsigned* bmax = p->tc_mode > 0 || gen_analysis(p) ? p->d_bmax : nullptr;
   if (e == cudaSuccess && bmax && p->tc_mode > 0) e = cudaMemsetAsync(bmax, 0, sizeof(unsigned) * p->nbatch, s);
   RingFork f(p, 0, s, e);
   Launch32 ls[4];

@@ -108,7 +108,8 @@ struct hpx_plan_s {
   int* d_gstart;       // [mmax+1][ngrid] earliest start of a group's chains
   float2* d_zf;        // [npair] z as a sum of two floats
   // generated-lambda tensor-core stages (hpx_gen.cu)
-  int gen_parts;       // 0: not used; 2: streamed split-product plans; 3: FP32 analysis in three BF16 parts
+  int gen_parts;       // 0: not used; 2: streamed split-product plans; 3: FP32 analysis in three BF16 parts,
+                       // where it pays (gen_analysis)
   int gen_nn;          // 3: N columns of the analysis products
   int gen_ctas;        // CTAs of the analysis (one per SM)
   float4* d_gen_state; // [gen_ctas][npair] chains between tiles
@@ -760,7 +761,12 @@ cudaError_t launch_synthesis_tc(hpx_plan_s* p, int b0, int nb, cudaStream_t s);
 // buffers build_gen makes), the synthesis At, as the table tiles do
 cudaError_t build_gen(hpx_plan_s* p, int parts, cudaStream_t s);
 size_t gen_extra_bytes_estimate(int nside, int mmax, int nbatch, int parts);
-int gen_parts_of(int nside, int nbatch, int dtype, unsigned flags);
+int gen_parts_of(int nside, int lmax, int mmax, int nbatch, int dtype, unsigned flags);
+bool gen_analysis_pays(int nside, int lmax, int mmax, int n);
+// whether this call's analysis (of p->nbatch channels, of a view fewer than the plan's) takes them
+inline bool gen_analysis(const hpx_plan_s* p) {
+  return p->gen_parts == 3 && gen_analysis_pays(p->nside, p->lmax, p->mmax, p->nbatch);
+}
 cudaError_t launch_pack_gen(hpx_plan_s* p, int b0, int nb, bool use_weight, cudaStream_t s);
 cudaError_t launch_gen_analysis(const hpx_plan_s* p, float* alm, double mfac, cudaStream_t s);
 cudaError_t launch_gen_synthesis(const hpx_plan_s* p, cudaStream_t s);

@@ -236,7 +236,7 @@ static cudaError_t run_analysis(hpx_plan_s* p, const void* map, void* alm, bool 
       });
     return e;
   }
-  if (p->gen_parts == 3) {
+  if (gen_analysis(p)) {
     // FP32 without tensor-core tables: the packs, then one launch that
     // generates lambda and contracts it for all channel groups
     const int cp = p->gen_nn / 4;
@@ -531,7 +531,7 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
     e = dtype == HPX_F64 ? build_lambda_table<double>(p, s) : build_lambda_table<float>(p, s);
   if (e == cudaSuccess && (flags & HPX_PLAN_TENSOR_CORES)) e = build_tc(p, s);
   if (e == cudaSuccess)
-    if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) e = build_gen(p, parts, s);
+    if (const int parts = gen_parts_of(nside, lmax, mmax, nbatch, dtype, flags)) e = build_gen(p, parts, s);
   if (e == cudaSuccess) e = f64 ? build_fft_tables<double>(p, s) : build_fft_tables<float>(p, s);
   if (e == cudaSuccess && tc1) e = build_fft_tables16(p, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
@@ -584,7 +584,7 @@ size_t hpx_plan_estimate_bytes(int nside, int lmax, int mmax, int nbatch, hpx_dt
     b += sizeof(RingInfo) * nring + cs * ((n16 ? n16 : 1) + ((size_t)1 << (logm_max - 1)) + (size_t)nside * (nside - 1));
   }
   if (has_starts32(dtype, mode, nbatch, nspec)) b += (sizeof(int) + sizeof(float4)) * nchain;
-  if (const int parts = gen_parts_of(nside, nbatch, dtype, flags)) b += gen_extra_bytes_estimate(nside, mmax, nbatch, parts);
+  if (const int parts = gen_parts_of(nside, lmax, mmax, nbatch, dtype, flags)) b += gen_extra_bytes_estimate(nside, mmax, nbatch, parts);
   if (flags & (HPX_PLAN_LAMBDA_HOST | HPX_PLAN_LAMBDA_STREAM))  // no resident table; two staging buffers
     return b + sizeof(int) +
            tc_extra_bytes_estimate(nside, lmax, mmax, nbatch, mode, true, (flags & HPX_PLAN_LAMBDA_STREAM) != 0);

@@ -1644,14 +1644,30 @@ cudaError_t launch_pack_tc(hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream
 // (three BF16 parts) where its cost, which hardly depends on the channels, is
 // below the CUDA-core kernel's for plans that recompute lambda and for those
 // that read the FP32 table (the two take one path, so that their results agree
-// bit for bit).  Analysis in ms, CUDA cores / tensor cores with the pack, at
-// lmax 3 Nside - 1, recomputing: Nside 256, 16 channels 0.64 / 0.43 (8: 0.32 /
-// 0.34); Nside 512, 8 channels 2.15 / 1.76; Nside 1024, 8 channels 15.7 / 10.6;
-// Nside 2048, 4 channels 137 / 76, 1 channel 52 / 75.
-int gen_parts_of(int nside, int nbatch, int dtype, unsigned flags) {
+// bit for bit).  The kernel gives a CTA one m, so a few m leave the chip idle
+// where the CUDA-core kernel's clusters of up to eight CTAs do not.  Whole
+// analyses in ms, CUDA cores / tensor cores, recomputing, lmax 3 Nside - 1:
+//   all m:      Nside 256, 8 channels 0.36 / 0.45, 12 0.69 / 0.47; Nside 512, 4 1.74 / 1.80,
+//               6 2.23 / 1.84; Nside 1024, 2 9.3 / 10.9, 4 12.8 / 10.9; Nside 2048, 2 60.6 /
+//               74.9, 3 137 / 75
+//   mmax 40:    Nside 512, 8 channels 0.36 / 0.47; Nside 1024, 8 1.01 / 1.54, 20 2.78 / 2.27;
+//               Nside 2048, 4 3.0 / 5.3
+//   mmax 75:    0.48 / 0.47; 1.41 / 1.55, 4.02 / 2.29; 5.5 / 5.4
+//   mmax 150:   0.66 / 0.47; 2.16 / 1.56, 6.25 / 3.82; 9.4 / 5.4
+// and at Nside 512, lmax 128, 8 channels 0.178 / 0.205, where the fixed costs decide.
+// At Nside 256, where those clusters are two CTAs, the tiles are no slower with few m or
+// l either (mmax 10, 12 channels 0.216 / 0.176; lmax 64 0.090 / 0.089).
+bool gen_analysis_pays(int nside, int lmax, int mmax, int n) {
+  const int from = nside >= 1024 ? 3 : nside >= 512 ? 5 : nside >= 256 ? 9 : INT_MAX;
+  if (n < from) return false;
+  return nside < 512 || (lmax >= 256 && (long long)(mmax + 1) * ((n + 7) / 8) >= 100);
+}
+// A plan has the operand for it from these channels on; narrower plans would pay its
+// memory for little.
+int gen_parts_of(int nside, int lmax, int mmax, int nbatch, int dtype, unsigned flags) {
   if (dtype != HPX_F32 || (flags & HPX_PLAN_TENSOR_CORES)) return 0;
   const int from = nside >= 2048 ? 4 : nside >= 512 ? 8 : nside >= 256 ? 12 : INT_MAX;
-  return nbatch >= from ? 3 : 0;
+  return nbatch >= from && gen_analysis_pays(nside, lmax, mmax, nbatch) ? 3 : 0;
 }
 
 static int gen_columns(int nbatch) { return tc_columns(nbatch, 16); }

@@ -175,6 +175,13 @@ int64_t hpx_nalm(int lmax, int mmax);
  * Builds the ring-geometry table, the recurrence coefficients, the starting
  * state of every (m, ring) recurrence chain and the FFT tables on the device;
  * returns once they are complete.  *out receives the plan.
+ * Wide HPX_F32 plans without HPX_PLAN_TENSOR_CORES (from 12 channels at Nside
+ * 256, 8 at 512 and 1024, 4 at 2048) also hold a tensor-core operand for their
+ * analyses: 24 bytes per m, ring pair and channel, 1.5 times their ring workspace,
+ * with the channels rounded up to 8 or a multiple of 16 (Nside 2048, lmax 6143, 4
+ * channels: 4.8 GB of 8.5).  Where the device has no room for it the plan is made
+ * without, and its analyses run on the CUDA cores (hpx_plan_device_bytes tells);
+ * both agree to FP32 rounding.
  * Errors: HPX_ERR_INVALID, HPX_ERR_NOMEM, HPX_ERR_CUDA, HPX_ERR_UNSUPPORTED. */
 hpx_status hpx_plan_create(int nside, int lmax, int mmax, int nbatch,
                            hpx_dtype dtype, hpx_plan* out);

@@ -1686,22 +1686,33 @@ cudaError_t build_gen(hpx_plan_s* p, int parts, cudaStream_t s) {
   p->gen_ctas = sms < 160 ? sms : 160;
   const size_t state = (size_t)p->gen_ctas * p->npair * sizeof(float4);
   e = cudaMalloc((void**)&p->d_gen_state, state);
-  if (e != cudaSuccess) return e;
-  p->bytes += state;
+  size_t maxima = 0, operand = 0;
   if (parts == 3) {
-    const size_t maxima = 2 * sizeof(unsigned) * (size_t)p->nbatch;
-    e = cudaMalloc((void**)&p->d_bmax, maxima);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_bmax, 0, maxima, s);
-    if (e != cudaSuccess) return e;
-    p->bytes += maxima;
-    p->bmax_stride = p->nbatch;
     const int nn = gen_columns(p->nbatch), rows = 3 * nn;
     p->gt_group_elems = (long long)(p->mmax + 1) * p->ngrid * rows * 64;
     p->gt_groups = (p->nbatch + nn / 4 - 1) / (nn / 4);
-    const size_t bytes = 2 * (size_t)p->gt_group_elems * p->gt_groups;
-    e = cudaMalloc(&p->d_gt, bytes);
+    maxima = 2 * sizeof(unsigned) * (size_t)p->nbatch;
+    operand = 2 * (size_t)p->gt_group_elems * p->gt_groups;
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_bmax, maxima);
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_gt, operand);
+    if (e == cudaErrorMemoryAllocation) {
+      // a plan that has no room for the operand keeps the CUDA-core analysis, which
+      // needs nothing beside the workspace
+      cudaGetLastError();
+      for (void** q : {(void**)&p->d_gen_state, (void**)&p->d_bmax, &p->d_gt}) {
+        if (*q) cudaFree(*q);
+        *q = nullptr;
+      }
+      return cudaSuccess;
+    }
+  }
+  if (e != cudaSuccess) return e;
+  p->bytes += state + maxima + operand;
+  if (parts == 3) {
+    const int nn = gen_columns(p->nbatch);
+    e = cudaMemsetAsync(p->d_bmax, 0, maxima, s);
     if (e != cudaSuccess) return e;
-    p->bytes += bytes;
+    p->bmax_stride = p->nbatch;
     if (!encode_rows128(p->tm_gt, p->d_gt, (unsigned long long)(p->gt_group_elems / 64) * p->gt_groups, nn, 2)) {
       set_error("cuTensorMapEncodeTiled failed or is unavailable");
       return cudaErrorInvalidValue;

@@ -154,13 +154,16 @@ typedef enum {
                                         lambda (Eq. 15-16).  Split-product
                                         plans (HPX_F32, HPX_F32_BF16X3,
                                         HPX_F32_FP16X3) generate it in shared
-                                        memory beside the products; the others
-                                        fill two device staging buffers, block
-                                        of m by block, on a second stream while
-                                        the tensor cores contract the other.
-                                        One recurrence serves up to 32 channels
-                                        (split products) or all of them.  Same
-                                        results as the resident plan.  Not with
+                                        memory beside the products; the others,
+                                        and analyses of more than 96 channels
+                                        (160 below Nside 512), fill two device
+                                        staging buffers, block of m by block,
+                                        on a second stream while the tensor
+                                        cores contract the other.  One
+                                        recurrence serves up to 32 channels in
+                                        shared memory, all of them from the
+                                        staging buffers.  Same results as the
+                                        resident plan.  Not with
                                         HPX_PLAN_LAMBDA_HOST. */
 
 /* Number of packed coefficients for (lmax, mmax). */
@@ -204,10 +207,14 @@ hpx_status hpx_plan_create_ooc(int nside, int lmax, int mmax, int nbatch,
 /* A streamed tensor-core plan (HPX_PLAN_LAMBDA_TABLE |
  * HPX_PLAN_TENSOR_CORES | HPX_PLAN_LAMBDA_STREAM, plus `flags`: 0 or
  * HPX_PLAN_TC_TF32X3 for an HPX_F32 plan) whose two device staging buffers
- * hold stage_bytes per table part (hi, and lo for the x3 dtypes); 0 selects
- * 1 GiB, or the larger table part where that is smaller.  dtype: HPX_F32 or a 16-bit dtype.  No table is built at plan
- * time.  HPX_ERR_INVALID for other flags or if one m's table slice does not
- * fit a staging buffer. */
+ * hold stage_bytes per table part (hi, and lo for split products); 0 selects
+ * 1 GiB, or the larger table part where that is smaller.  dtype: HPX_F32 or a
+ * 16-bit dtype.  No table is built at plan time.  Split-product plans have
+ * the buffers only where nbatch is above the channels from which their
+ * analyses use them (see HPX_PLAN_LAMBDA_STREAM), and do without them if the
+ * device has no room; a call that is being captured never uses them there.
+ * HPX_ERR_INVALID for other flags or, with or without the buffers, if one m's
+ * table slice does not fit stage_bytes. */
 hpx_status hpx_plan_create_stream(int nside, int lmax, int mmax, int nbatch,
                                   hpx_dtype dtype, unsigned flags,
                                   size_t stage_bytes, hpx_plan* out);

@@ -111,6 +111,10 @@ struct hpx_plan_s {
   int gen_parts;       // 0: not used; 2: streamed split-product plans; 3: FP32 analysis in three BF16 parts,
                        // where it pays (gen_analysis)
   int gen_nn;          // 3: N columns of the analysis products
+  int gen_wide;        // 2: N columns of the table tiles that wide analyses take instead, their lambda
+                       // staged (0: no staging buffers); their operand in d_gt likewise
+  long long gt_group_elems_wide;
+  alignas(64) unsigned char tm_gt_wide[128];
   int gen_ctas;        // CTAs of the analysis (one per SM)
   float4* d_gen_state; // [gen_ctas][npair] chains between tiles
   void* d_spec;        // workspace [nbatch][nspec] C2<T>
@@ -767,6 +771,8 @@ bool gen_analysis_pays(int nside, int lmax, int mmax, int n);
 inline bool gen_analysis(const hpx_plan_s* p) {
   return p->gen_parts == 3 && gen_analysis_pays(p->nside, p->lmax, p->mmax, p->nbatch);
 }
+// the plan as the staged wide analysis of a streamed split-product plan sees it; false if this call does not take it
+bool staged_view(const hpx_plan_s* p, cudaStream_t s, hpx_plan_s* view);
 cudaError_t launch_pack_gen(hpx_plan_s* p, int b0, int nb, bool use_weight, cudaStream_t s);
 cudaError_t launch_gen_analysis(const hpx_plan_s* p, float* alm, double mfac, cudaStream_t s);
 cudaError_t launch_gen_synthesis(const hpx_plan_s* p, cudaStream_t s);

@@ -210,6 +210,26 @@ static cudaError_t staged(hpx_plan_s* p, int stage, cudaStream_t s, F&& f) {
   return e != cudaSuccess ? e : e2;
 }
 
+// The analysis' Legendre stage on tensor-core plans: the operand pack of every
+// channel group (stage 4), then one tile launch over all groups (stage 1).
+static cudaError_t run_tc_analysis(hpx_plan_s* p, void* alm, bool weighted, double mfac, cudaStream_t s) {
+  const int cp = tc_channels_per_launch(p, false);
+  cudaError_t e = cudaSuccess;
+  for (int b0 = 0; b0 < p->nbatch && e == cudaSuccess; b0 += cp) {
+    const int nb = p->nbatch - b0 < cp ? p->nbatch - b0 : cp;
+    e = staged(p, 4, s, [&](int* n) {
+      *n = 1;
+      return launch_pack_tc(p, b0, nb, weighted, s);
+    });
+  }
+  if (e == cudaSuccess)
+    e = staged(p, 1, s, [&](int* n) {
+      *n = 1;
+      return launch_tile_tc(p, static_cast<float*>(alm), 0, p->nbatch, mfac, s);
+    });
+  return e;
+}
+
 template <typename T>
 static cudaError_t run_analysis(hpx_plan_s* p, const void* map, void* alm, bool weighted, double mfac,
                                 cudaStream_t s) {
@@ -218,24 +238,13 @@ static cudaError_t run_analysis(hpx_plan_s* p, const void* map, void* alm, bool 
     return launch_r2c<T>(p, static_cast<const T*>(map), s);
   });
   if (e != cudaSuccess) return e;
-  if (p->tc_nn_a) {
-    // tensor cores: the operand pack of every channel group (stage 4), then
-    // one tile launch over all groups (stage 1)
-    const int cp = tc_channels_per_launch(p, false);
-    for (int b0 = 0; b0 < p->nbatch && e == cudaSuccess; b0 += cp) {
-      const int nb = p->nbatch - b0 < cp ? p->nbatch - b0 : cp;
-      e = staged(p, 4, s, [&](int* n) {
-        *n = 1;
-        return launch_pack_tc(p, b0, nb, weighted, s);
-      });
-    }
-    if (e == cudaSuccess)
-      e = staged(p, 1, s, [&](int* n) {
-        *n = 1;
-        return launch_tile_tc(p, static_cast<float*>(alm), 0, p->nbatch, mfac, s);
-      });
+  hpx_plan_s view;
+  if (staged_view(p, s, &view)) {
+    e = run_tc_analysis(&view, alm, weighted, mfac, s);
+    p->stage_next = view.stage_next;
     return e;
   }
+  if (p->tc_nn_a) return run_tc_analysis(p, alm, weighted, mfac, s);
   if (gen_analysis(p)) {
     // FP32 without tensor-core tables: the packs, then one launch that
     // generates lambda and contracts it for all channel groups

@@ -1317,7 +1317,8 @@ static_assert(kSynChannels == 8 || kSynChannels == 16 || kSynChannels == 32, "sy
 constexpr int kSynChannelsFK = HPX_TC_SYN_CHANNELS_FK;
 // Channels per CTA of the tiles that generate their lambda (streamed
 // split-product plans): up to 32, whose operand tiles leave room for the
-// lambda tiles; wider transforms run the recurrence once per 32.
+// lambda tiles; wider transforms run the recurrence once per 32 (analyses of many
+// more are staged, staged_analysis_pays).
 constexpr int kGenChannels = 32;
 static_assert(kSynChannelsFK == 32 || kSynChannelsFK == 64, "single-product synthesis channel group");
 
@@ -1334,6 +1335,14 @@ static int syn_channels(int mode, bool streamed) {
 }
 static int ana_channels(int mode, bool streamed) { return mode == 0 ? 32 : mode == 2 && streamed ? kGenChannels : kAnaChannels; }
 
+// Streamed split-product analyses of many channels: the generated tiles rerun the
+// recurrence for every 32, a staged fill serves all of them and its tiles take 64.
+// Analysis in ms, generated / staged, lmax 3 Nside - 1 (Nside 1024: 2047): Nside 256,
+// 96 channels 1.29 / 1.52, 128 1.68 / 1.72, 160 2.08 / 2.24, 192 2.48 / 2.45; Nside 512, 96 5.95 /
+// 6.80, 97 7.42 / 6.83, 160 9.75 / 9.79, 192 11.7 / 10.5; Nside 1024, 96 18.4 / 19.7, 97 23.0 /
+// 19.8, 160 30.4 / 28.0; Nside 2048, 96 223 / 237, 128 296 / 249.
+static bool staged_analysis_pays(int nside, int n) { return n > (nside >= 512 ? 96 : 160); }
+
 size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mode, bool host_tables, bool streamed) {
   if (mode < 0) return 0;
   const size_t es = mode ? 2 : 4, kw = mode ? 64 : 32, parts = mode == 2 ? 2 : 1;
@@ -1347,14 +1356,17 @@ size_t tc_extra_bytes_estimate(int nside, int lmax, int mmax, int nbatch, int mo
   }
   const size_t cps = nns / 4, groups = ((size_t)nbatch + cps - 1) / cps;
   const size_t cpa = nna / 4, groups_a = ((size_t)nbatch + cpa - 1) / cpa;
-  size_t b = es * (size_t)(mmax + 1) * ngroup * nna * kw * parts * groups_a  // Gt, one region per channel group
+  const bool wide = mode == 2 && streamed && staged_analysis_pays(nside, nbatch);
+  const size_t gt_rows = wide ? std::max(nna * groups_a, (size_t)(4 * kAnaChannels) * (((size_t)nbatch + kAnaChannels - 1) / kAnaChannels))
+                              : nna * groups_a;
+  size_t b = es * (size_t)(mmax + 1) * ngroup * kw * parts * gt_rows         // Gt, one region per channel group
              + es * chunks * nns * kw * parts * groups                       // At, likewise
              + (sizeof(int) + sizeof(long long)) * (size_t)(mmax + 1) * (nptile + ngroup) +
              sizeof(long long) * (mmax + 2) + 2 * sizeof(unsigned) * nbatch;
   const size_t col = es * chunks * nptile * 128 * kw, row = es * rows * ngroup * kw;  // upper bounds, a part
-  if (mode == 2 && streamed) return b + gen_extra_bytes_estimate(nside, mmax, nbatch, 2);  // nothing staged
-  if (host_tables)  // staging buffers at the default size
-    return b + 2 * parts * std::min(size_t(1) << 30, (std::max(col, row) + 127) / 128 * 128);
+  const size_t staging = 2 * parts * std::min(size_t(1) << 30, (std::max(col, row) + 127) / 128 * 128);  // default size
+  if (mode == 2 && streamed) return b + gen_extra_bytes_estimate(nside, mmax, nbatch, 2) + (wide ? staging : 0);
+  if (host_tables) return b + staging;
   b += parts * col;           // column table
   if (mode) b += parts * row;  // 16-bit row table
   return b;
@@ -1479,10 +1491,24 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
     e = cudaMemcpy(p->d_tab_off, roff.data(), sizeof(long long) * nent, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
   }
-  // analysis operand, one region per channel group
+  // analysis operand, one region per channel group; of both widths where wide
+  // calls are staged
   p->gt_group_elems = (long long)(p->mmax + 1) * p->ngroup * rba * kw;
   p->gt_groups = (p->nbatch + nna / 4 - 1) / (nna / 4);
-  e = dalloc(&p->d_gt, (size_t)es * p->gt_group_elems * p->gt_groups);
+  const size_t gt_bytes = (size_t)es * p->gt_group_elems * p->gt_groups;
+  const int groups_wide = (p->nbatch + kAnaChannels - 1) / kAnaChannels;
+  size_t gt_wide_bytes = 0;
+  if (mode == 2 && streamed && staged_analysis_pays(p->nside, p->nbatch)) {
+    p->gen_wide = 4 * kAnaChannels;
+    p->gt_group_elems_wide = (long long)(p->mmax + 1) * p->ngroup * 2 * p->gen_wide * kw;
+    gt_wide_bytes = (size_t)es * p->gt_group_elems_wide * groups_wide;
+  }
+  e = dalloc(&p->d_gt, std::max(gt_bytes, gt_wide_bytes));
+  if (e == cudaErrorMemoryAllocation && gt_wide_bytes > gt_bytes) {
+    cudaGetLastError();
+    p->gen_wide = 0;
+    e = dalloc(&p->d_gt, gt_bytes);
+  }
   if (e != cudaSuccess) return e;
   // synthesis operand: chunk offsets of each m, then At
   std::vector<long long> ach(p->mmax + 2);
@@ -1565,8 +1591,19 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
     std::copy(rbb.begin(), rbb.end(), p->blk_row_base);
     std::copy(cbb.begin(), cbb.end(), p->blk_col_base);
     if (streamed && mode == 2) e = build_gen(p, 2, s);  // lambda never leaves the kernels
-    const bool staged = p->gen_parts != 2;
+    bool staged = p->gen_parts != 2 || p->gen_wide;
     for (int b = 0; b < 2 && e == cudaSuccess && staged; ++b) e = dalloc(&p->d_stage[b], p->stage_bytes * parts);
+    if (e == cudaErrorMemoryAllocation && p->gen_wide) {  // no room: wide analyses take the generated tiles too
+      cudaGetLastError();
+      if (p->d_stage[0]) {
+        cudaFree(p->d_stage[0]);
+        p->bytes -= p->stage_bytes * parts;
+      }
+      p->d_stage[0] = p->d_stage[1] = nullptr;
+      p->gen_wide = 0;
+      staged = false;
+      e = cudaSuccess;
+    }
     if (e != cudaSuccess) return e;
     if (host) {
       auto halloc = [&](void** ptr, size_t bytes) -> cudaError_t {
@@ -1607,17 +1644,21 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
         return cudaErrorInvalidValue;
       }
     }
-    cudaStream_t cs;
-    e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    p->copy_stream = cs;
-    cudaEvent_t* ev = new cudaEvent_t[4]();
-    p->stage_events = ev;
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
-    if (e != cudaSuccess) return e;
+    if (staged) {
+      cudaStream_t cs;
+      e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+      if (e != cudaSuccess) return e;
+      p->copy_stream = cs;
+      cudaEvent_t* ev = new cudaEvent_t[4]();
+      p->stage_events = ev;
+      for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+      if (e != cudaSuccess) return e;
+    }
   }
   if (!encode_rows128(p->tm_gt, p->d_gt, (unsigned long long)(p->mmax + 1) * p->ngroup * rba * p->gt_groups, nna,
                       es) ||
+      (p->gen_wide && !encode_rows128(p->tm_gt_wide, p->d_gt, (unsigned long long)(p->gt_group_elems_wide / kw) * groups_wide,
+                                      p->gen_wide, es)) ||
       !encode_rows128(p->tm_at, p->d_at, (unsigned long long)ach[p->mmax + 1] * rbs * p->at_groups, nns, es)) {
     set_error("cuTensorMapEncodeTiled failed or is unavailable");
     return cudaErrorInvalidValue;
@@ -1625,6 +1666,24 @@ cudaError_t build_tc(hpx_plan_s* p, cudaStream_t s) {
   p->tc_nn_a = nna;
   p->tc_nn_s = nns;
   return cudaSuccess;
+}
+
+// A call that is being captured keeps to its stream, as the generated tiles do: the
+// staging buffers' events would tie the capture to work outside it.
+bool staged_view(const hpx_plan_s* p, cudaStream_t s, hpx_plan_s* view) {
+  if (!p->gen_wide || !staged_analysis_pays(p->nside, p->nbatch)) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return false;
+  *view = *p;
+  view->gen_parts = 0;
+  view->tc_nn_a = p->gen_wide;
+  view->gt_group_elems = p->gt_group_elems_wide;
+  std::copy(p->tm_gt_wide, p->tm_gt_wide + sizeof(p->tm_gt_wide), view->tm_gt);
+  return true;
 }
 
 cudaError_t launch_pack_tc(hpx_plan_s* p, int b0, int nb, bool use_w, cudaStream_t s) {

@@ -40,11 +40,14 @@ SEED = 2510017850 + 2
 # FP64 peak from unit counts and clocks: 152 SMs x 2 FP64 FMA/clk/SM x
 # 2 flop x 2.07 GHz (the published 1.25 TFLOP/s dense FP64 of a GB300).
 # FP32 pipe operations per second (152 SMs x 128 lanes x 2.07 GHz), the bound
-# of the recomputing FP32 kernels, whose recurrence runs in double-FP32
+# of the recomputing FP32 kernels
 FP32_OPS_PEAK = 152 * 128 * 2.070e9 / 1e12
 # FP32 operations of one double-FP32 recurrence step (the product c_l z: 4;
-# times mu_{l-1}: 4; the TwoSum with mu_{l-2}: 6; error terms: 2; FastTwoSum: 3)
+# times mu_{l-1}: 4; the TwoSum with mu_{l-2}: 6; error terms: 2; FastTwoSum: 3),
+# in which a recomputing stage's work is counted; and of a grid step, which the
+# kernels take for four values in five and more: what they execute at least
 DF_STEP_OPS = 19
+GRID_STEP_OPS = 12
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 
 
@@ -429,8 +432,10 @@ def run_ours(args):
     rec["accuracy"] = plan_accuracy(plan_r, maps, alm_in, ref64)
     plan_r.close()
 
-    # plan-resident lambda table (built by the same double-FP32 recurrence at
-    # plan time), Legendre analysis on the CUDA cores
+    # plan-resident FP32 lambda table (built by the same recurrence at plan
+    # time) without tensor-core tables: synthesis on the CUDA cores, and the
+    # analysis too below 8 channels (from there in three BF16 parts, its tiles
+    # filled from the table)
     plan_c = hpx.Plan(NSIDE, LMAX, MMAX, NBATCH, "f32", lambda_table=True, device=dev)
     cc = timed_steps(plan_c, maps, alm_in, args, dist, dev, world, gpu_index)
     cc["roofline"] = legendre_roofline(plan_c, cc["stages"], table=True)
@@ -522,7 +527,9 @@ def run_ours(args):
                 "lambda_recompute": {k: rec[k] for k in ("value", "roofline", "stages", "accuracy", "clocks")}
                 | {"ms_per_step": rec["t_max"] / args.steps}}
         for k in ("tensor_core_tf32x3", "cuda_core_table", "lambda_recompute"):
-            note(f"{k}: {line[k]['value']:.1f} pairs/s, roofline frac {line[k]['roofline']['frac']:.3f}")
+            r = line[k]["roofline"]
+            note(f"{k}: {line[k]['value']:.1f} pairs/s, {r['kernel']} roofline frac {r['frac']:.3f}"
+                 + (f" ({r['frac_executed']:.3f} of the operations executed)" if "frac_executed" in r else ""))
         emit(line, args.record)
     plan.close()
     if dist.is_available() and dist.is_initialized():
@@ -602,8 +609,10 @@ def legendre_roofline(plan, stages, table: bool, value_bytes: int = 4):
     """Roofline of the slower Legendre kernel, with per-stage figures added
     to `stages` in place.
 
-    Recomputing plans: the FP64 pipe, 3 flop per significant (l, m,
-    ring-pair) triple (one DMUL + one DFMA per step of the recurrence).
+    Recomputing plans: the FP32 pipe, a double-FP32 recurrence step and 2 FMA
+    per channel for every significant (l, m, ring-pair) triple; the figures
+    named executed count the grid step, and no FMAs where the products run on
+    the tensor cores (wide analyses).
     Table plans: HBM, algorithmic bytes only: `value_bytes` per significant
     triple (4 for FP32 and for FP16 hi/lo pairs, 2 for one 16-bit part) plus
     the stage's own input and output (analysis: half spectra in, alm out;
@@ -623,6 +632,8 @@ def legendre_roofline(plan, stages, table: bool, value_bytes: int = 4):
         if k in stages and stages[k]["ms_per_step"] > 0:
             s = stages[k]
             s["hbm_gbs_algorithmic"] = by / (s["ms_per_step"] / 1e3) / 1e9
+    tc = "analysis_operand_pack" in stages
+    gen = tc and plan.column_table_bytes == 0  # a wide analysis of a plan without tensor-core tables
     lam_bytes = value_bytes * active if table else 0
     leg_io = {"legendre_analysis": spec_bytes + alm_bytes, "legendre_synthesis": alm_bytes + f_bytes}
     for k in ("legendre_analysis", "legendre_synthesis"):
@@ -633,12 +644,13 @@ def legendre_roofline(plan, stages, table: bool, value_bytes: int = 4):
             s["hbm_gbs_algorithmic"] = (lam_bytes + leg_io[k]) / sec / 1e9
         else:  # the recurrence step plus 2 FMA per channel (complex times real) per triple
             s["fp32_pipe_tops"] = (DF_STEP_OPS + 2 * NBATCH) * active / sec / 1e12
+            fma = 0 if gen and k == "legendre_analysis" else 2 * NBATCH
+            s["fp32_pipe_tops_executed"] = (GRID_STEP_OPS + fma) * active / sec / 1e12
     dom = max(["legendre_analysis", "legendre_synthesis"], key=lambda k: stages[k]["ms_per_step"])
-    tc = "analysis_operand_pack" in stages
     side = "analysis" if dom == "legendre_analysis" else "synthesis"
-    kname = f"k_legendre_{side}"
+    kname = f"k_gen_{side}" if gen and side == "analysis" else f"k_legendre_{side}"
     if table:
-        kname = f"k_legendre_tc<{side}>" if tc else kname + "<table>"
+        kname = f"k_legendre_tc<{side}>" if tc and not gen else kname + "<table>"
         achieved = stages[dom]["hbm_gbs_algorithmic"]
         return {"bound": "hbm", "kernel": kname, "achieved": achieved, "peak": HBM_PEAK_GBS,
                 "unit": "GB/s", "frac": achieved / HBM_PEAK_GBS, "traffic": kernel_traffic(kname),
@@ -648,20 +660,21 @@ def legendre_roofline(plan, stages, table: bool, value_bytes: int = 4):
     return {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": FP32_OPS_PEAK,
             "unit": "TOP/s", "frac": achieved / FP32_OPS_PEAK, "traffic": kernel_traffic(kname),
             "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz",
+            "frac_executed": stages[dom]["fp32_pipe_tops_executed"] / FP32_OPS_PEAK,
             "work": f"({DF_STEP_OPS} + 2 x {NBATCH}) FP32 operations x {active} significant (l,m,ring-pair) "
-                    f"triples per step (of {total}; contributions below 2^-193 dropped): a double-FP32 "
-                    f"recurrence step and 2 FMA per channel"}
+                    f"triples per step (of {total}; values below 2^-136 are zero in FP32): a double-FP32 "
+                    f"recurrence step and 2 FMA per channel; executed: {GRID_STEP_OPS} a grid step"}
 
 
 SERVE_MIX = {64: 0.30, 128: 0.25, 256: 0.20, 512: 0.15, 1024: 0.07, 2048: 0.03}
 # slots with a plan-time lambda table on the tensor cores, and slots that
-# recompute lambda per batch into streamed blocks contracted on the tensor
-# cores (one recurrence per batch, whatever its channels); channels per
-# batch: one table stream or one recurrence serves every request of a batch
+# recompute lambda per batch beside the products on the tensor cores (one
+# recurrence per 32 channels); channels per batch: one pass over the table,
+# or over the recurrences, serves every request of a batch
 SERVE_TABLE_NSIDES = (64, 128, 256)
 SERVE_STREAMED_NSIDES = (512, 1024, 2048)
 # (all six slots resident under the cap: the Nside-1024 table slot alone
-# held 74 GB, and a streamed Nside-2048 slot of 32 channels about 59 GB)
+# held 74 GB)
 SERVE_BATCH = {64: 64, 128: 64, 256: 64, 512: 64, 1024: 64, 2048: 32}
 
 

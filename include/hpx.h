@@ -17,7 +17,9 @@
  *
  * with lambda_lm the orthonormal associated Legendre functions including the
  * Condon-Shortley phase (Eq. 8, 15), generated by the three-term recurrence
- * in l (Eq. 16) in FP64, and equal-area weights w_y = 4 pi / Npix (Eq. 1).
+ * in l (Eq. 16) -- in FP64 for HPX_F64 plans, in FP32 pairs of at least 39
+ * significant bits for the others, whose error is at most about that of
+ * rounding the values to FP32 -- and equal-area weights w_y = 4 pi / Npix (Eq. 1).
  *
  * Data layout (all device buffers are owned by the caller):
  *   map : [nbatch][12 nside^2] real, RING order (rings north to south,
@@ -70,12 +72,14 @@ typedef struct hpx_plan_s* hpx_plan;
 
 /* I/O precision and contraction mode.
  *   HPX_F64        double maps/coefficients, FP64 contraction.
- *   HPX_F32        float maps/coefficients, FP32 contraction; lambda_lm still
- *                  comes from the FP64 recurrence.
+ *   HPX_F32        float maps/coefficients, FP32 lambda_lm and contraction to
+ *                  FP32 accuracy: on the CUDA cores, or as split products on
+ *                  the tensor cores (wide analyses in three BF16 parts, see
+ *                  hpx_plan_create; HPX_PLAN_TENSOR_CORES).
  *   HPX_F32_BF16 / HPX_F32_FP16     float I/O (ring transforms in FP32);
  *                  both Legendre stages on tensor cores from plan-resident
- *                  BF16 / FP16 lambda tables (rounded from the FP64
- *                  recurrence) and BF16 / FP16 operands, FP32 accumulation.
+ *                  BF16 / FP16 lambda tables (rounded from the FP32
+ *                  values) and BF16 / FP16 operands, FP32 accumulation.
  *                  FP16 operands are scaled per channel by a power of two
  *                  (from the largest component of the channel's spectra or
  *                  coefficients) to stay in range; the scale is undone on

@@ -8,7 +8,8 @@
 //   k_gen_synthesis  D[p][n] = sum_l Lambda[l][p] At[n][l], a CTA 128 pairs of
 //                    four m
 //
-// Used by the streamed-lambda plans of the split-product modes (two 16-bit
+// Used by the streamed-lambda plans of the split-product modes (all syntheses, and
+// analyses of up to 96 or 160 channels, staged_analysis_pays; two 16-bit
 // parts, three products: the same values, products and sums as the table
 // tiles, so the same bits), and by the analysis of the FP32 plans without
 // tensor-core tables, in three BF16 parts and six products: 3 x 8 significant

@@ -653,7 +653,7 @@ struct Chains2 {
 // every group g of 32 consecutive ring pairs, rows l = lstart(m,g)..lmax of 32
 // values mu_l (one per pair of the group), lstart = the group's earliest chain
 // start; row r of (m, g) at tab[off(m,g) + 32 r].  Written once at plan time
-// by the same FP64 recurrence and conversion as the recomputing kernels.
+// by the steps of the recomputing kernels (FP64 plans RecurD, the others Chain).
 template <typename T> struct LamTab {
   const T* tab;
   const long long* off;

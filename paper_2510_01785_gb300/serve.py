@@ -221,11 +221,11 @@ class GpuExecutor:
     table_nsides: geometries whose slots hold a plan-time lambda table on the
     tensor cores (FP16 hi/lo split products, FP32 accuracy); streamed_nsides:
     geometries whose slots recompute lambda per call beside the products on
-    the tensor cores (no table held; one recurrence per
-    batch whatever its channel count); the others recompute lambda on the
-    CUDA cores, once per group of channels of a launch.
+    the tensor cores (no table held; one recurrence per 32 channels of a
+    batch); the others recompute lambda on the CUDA cores, once per group of
+    channels of a launch.
     batch_channels: channels per batch by Nside (default 32); one batch runs
-    the recurrence, or streams the table, once for all its requests."""
+    those recurrences, or streams the table, once for all its requests."""
 
     def __init__(self, device=None, keep_outputs: bool = True, lambda_table_nsides=(), batch_channels=None,
                  tensor_cores: bool = True, streamed_nsides=()):

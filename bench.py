@@ -509,7 +509,7 @@ def run_ours(args):
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None, "dtype": "f32",
-                "precision": "FP32 I/O; lambda from the double-FP32 recurrence (plan-time table); contraction on "
+                "precision": "FP32 I/O; lambda from a recurrence in FP32 pairs (plan-time table); contraction on "
                              "tcgen05 as FP16 hi/lo split products (hi*hi + hi*lo + lo*hi, FP32 sums): "
                              f"{acc['map2alm_max_rel_l2_vs_f64']:.1e} / {acc['alm2map_max_rel_l2_vs_f64']:.1e} "
                              "rel. L2 vs FP64",

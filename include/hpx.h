@@ -37,7 +37,10 @@
  * of its kernels onto a plan-owned second stream (one for analyses, one for
  * syntheses) and joins it back before the call's next work on the caller's
  * stream, so the call stays ordered there and a stream capture records the
- * fork and the join.  A plan owns device workspace: one part for its
+ * fork and the join; on a stream with a priority of its own everything stays
+ * there.  Kernels of large transforms fill every SM for up to tens of
+ * milliseconds: calls that are to overtake them need a stream of higher
+ * priority.  A plan owns device workspace: one part for its
  * analyses (hpx_map2alm, hpx_alm2map_adjoint, hpx_map2alm_n) and one for
  * its syntheses (hpx_alm2map, hpx_map2alm_adjoint, hpx_alm2map_n).  So one
  * analysis and one synthesis may run at the same time on two streams

@@ -687,6 +687,14 @@ struct RingFork {
   cudaEvent_t join_ev = nullptr;
   RingFork(const hpx_plan_s* p, int which, cudaStream_t s_, cudaError_t& e) : s(s_), side(s_) {
     if (!p->fft_streams || p->nside < kRingSplitNside || e != cudaSuccess) return;
+    // a stream with a priority of its own keeps all its launches: on the second
+    // stream, of default priority, the belt rings would wait behind the work that
+    // the caller's is to overtake
+    int prio = 0;
+    if (cudaStreamGetPriority(s, &prio) != cudaSuccess || prio != 0) {
+      cudaGetLastError();
+      return;
+    }
     cudaStream_t st = static_cast<cudaStream_t*>(p->fft_streams)[which];
     cudaEvent_t* ev = static_cast<cudaEvent_t*>(p->fft_events) + 2 * which;
     e = cudaEventRecord(ev[0], s);

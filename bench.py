@@ -985,7 +985,7 @@ def run_small_configs(dev) -> dict:
         diff[f"nside{ns}_lmax{lmax}_b{nb}"] = {
             "loss1_forward_backward_ms": _event_ms(loss1, dev, reps, 1),
             "loss2_forward_backward_ms": _event_ms(loss2, dev, reps, 1),
-            "dtype": "f32", "lambda": "recomputed by the double-FP32 recurrence in forward and backward"}
+            "dtype": "f32", "lambda": "recomputed in forward and backward"}
         del maps, alm, target, ell, wl
         hpx.clear_plans()
         torch.cuda.empty_cache()

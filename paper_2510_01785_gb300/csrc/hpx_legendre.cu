@@ -103,15 +103,18 @@ __global__ void k_recurrence_coefs(int lmax, int mmax, double* coef_c, double* c
 
 // Start of every chain (m, pair): the first l at which |mu_l| >= 2^-sig,
 // with (mu_{l-1}, mu_l) there; l_c = lmax + 1 if the chain never gets there.
-// FP32 plans (lgrid, where given, zeroed before): also, per group of 64 pairs, the
+// FP32 plans (lgrid given, zeroed before): also, per group of 64 pairs, the
 // largest over its chains of the first l past l_c at which |mu_l| >=
 // 2^-kGridExp (lmax + 1 where a chain never gets there; a plain FP32
 // recurrence finds it), and in gstart (large before) the earliest l_c.
+// lc32 and start32, where given: the start from 2^-sig; lc_tab, start and the groups
+// then are of the later one, 2^-sig2 (the same values on the way: scaling by powers
+// of two is exact).
 __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* __restrict__ cmm,
                              const double* __restrict__ coef_c, const float2* __restrict__ coef_cf, int lmax,
-                             int npair, int sig, int* lc_tab, double* mu0_tab, double* mu1_tab,
+                             int npair, int sig, int sig2, int* lc_tab, double* mu0_tab, double* mu1_tab,
                              float4* __restrict__ start, int* __restrict__ lgrid, int* __restrict__ gstart,
-                             int ngrid) {
+                             int ngrid, int* __restrict__ lc32, float4* __restrict__ start32) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (p >= npair) return;
@@ -154,6 +157,23 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
   }
   const long long ci = (long long)m * npair + p;
   if (k > 0) mu1 = mu2 = 0.0;
+  if (lc32) {
+    lc32[ci] = k > 0 ? lmax + 1 : l;
+    const Df d0 = df_of(mu2 * kDfUp), d1 = df_of(mu1 * kDfUp);
+    start32[ci] = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
+    const double up2 = ldexp(1.0, -sig2);
+    while (k <= 0 && fabs(mu1) < up2) {
+      if (l == lmax) {
+        k = 1;  // never gets there
+        mu1 = mu2 = 0.0;
+        break;
+      }
+      ++l;
+      const double mu = fma(coef_c[base + l] * z, mu1, -mu2);
+      mu2 = mu1;
+      mu1 = mu;
+    }
+  }
   lc_tab[ci] = k > 0 ? lmax + 1 : l;
   if (!start) {
     mu0_tab[ci] = mu2;
@@ -162,7 +182,6 @@ __global__ void k_chain_scan(const RingInfo* __restrict__ rings, const double* _
   }
   const Df d0 = df_of(mu2 * kDfUp), d1 = df_of(mu1 * kDfUp);
   start[ci] = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
-  if (!lgrid) return;
   int lg = lmax + 1;
   if (k <= 0 && !grid_never(p & ~63, npair, lmax)) {
     const float zf = (float)z;
@@ -657,7 +676,7 @@ cudaError_t build_recurrence_tables(hpx_plan_s* p, cudaStream_t s) {
   k_coef_pairs<<<(unsigned)(nb < 4096 ? nb : 4096), 256, 0, s>>>(p->d_coef_c, p->d_coef_cf, p->nalm);
   const int mode = tc_mode_of(p->dtype, p->flags);
   const bool half = mode > 0 && p->dtype != HPX_F32_BF16 && p->dtype != HPX_F32_BF16X3;
-  const int sig = p->dtype == HPX_F64 ? kSigExp64 : half ? kSigExpHalf : kSigExp32;
+  const int sig = p->dtype == HPX_F64 ? kSigExp64 : half && !p->d_lc32 ? kSigExpHalf : kSigExp32;
   if (p->d_lgrid) {
     const size_t bytes = sizeof(int) * (size_t)(p->mmax + 1) * p->ngrid;
     cudaError_t e = cudaMemsetAsync(p->d_lgrid, 0, bytes, s);
@@ -666,12 +685,8 @@ cudaError_t build_recurrence_tables(hpx_plan_s* p, cudaStream_t s) {
     k_z_pairs<<<(p->npair + 127) / 128, 128, 0, s>>>(p->d_ring, p->d_zf, p->npair);
   }
   k_chain_scan<<<dim3((p->npair + 127) / 128, p->mmax + 1), 128, 0, s>>>(
-      p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, sig, p->d_lc, p->d_mu0, p->d_mu1, p->d_start,
-      p->d_lgrid, p->d_gstart, p->ngrid);
-  if (p->d_lc32)
-    k_chain_scan<<<dim3((p->npair + 127) / 128, p->mmax + 1), 128, 0, s>>>(
-        p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, kSigExp32, p->d_lc32, nullptr, nullptr,
-        p->d_start32, nullptr, nullptr, p->ngrid);
+      p->d_ring, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->lmax, p->npair, sig, half ? kSigExpHalf : sig, p->d_lc, p->d_mu0,
+      p->d_mu1, p->d_start, p->d_lgrid, p->d_gstart, p->ngrid, p->d_lc32, p->d_start32);
   return cudaGetLastError();
 }
 

@@ -156,7 +156,7 @@ static void plan_free(hpx_plan_s* p) {
     delete[] st;
   }
   void* ptrs[] = {p->d_ring, p->d_etab, p->d_btab, p->d_chirp, p->d_tw, p->d_ring16, p->d_btab16, p->d_chirp16, p->d_tw16, p->d_cmm, p->d_coef_c, p->d_coef_cf, p->d_coef_p,
-                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_lc32, p->d_start32, p->d_coef_pp, p->d_lgrid, p->d_gstart, p->d_zf,
+                  p->d_coef_pf, p->d_lc, p->d_mu0, p->d_mu1, p->d_start, p->d_coef_pp, p->d_lgrid, p->d_gstart, p->d_zf,
                   p->d_gen_state, p->d_spec, p->d_F, p->d_io_map, p->d_io_alm,
                   p->d_tab, p->d_tab_off, p->d_tab_lstart, p->d_gt, p->d_status, p->d_at, p->d_achunk,
                   p->d_stab, p->d_stab_off, p->d_stab_lstart, p->d_tab_lo, p->d_stab_lo, p->d_bmax,
@@ -490,20 +490,22 @@ static hpx_status create_plan(int nside, int lmax, int mmax, int nbatch, hpx_dty
             (f64 ? alloc((void**)&p->d_coef_p, sizeof(double) * p->nalm)
                  : alloc((void**)&p->d_coef_pp, sizeof(float2) * p->nalm)) &&
             alloc((void**)&p->d_coef_pf, sizeof(float) * p->nalm) &&
-            alloc((void**)&p->d_lc, sizeof(int) * nchain) &&
+            alloc((void**)&p->d_lc, sizeof(int) * nchain * (starts32 ? 2 : 1)) &&
             (f64 ? alloc((void**)&p->d_mu0, sizeof(double) * nchain) && alloc((void**)&p->d_mu1, sizeof(double) * nchain)
-                 : alloc((void**)&p->d_start, sizeof(float4) * nchain) &&
+                 : alloc((void**)&p->d_start, sizeof(float4) * nchain * (starts32 ? 2 : 1)) &&
                        alloc((void**)&p->d_lgrid, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
                        alloc((void**)&p->d_gstart, sizeof(int) * (size_t)(mmax + 1) * p->ngrid) &&
                        alloc((void**)&p->d_zf, sizeof(float2) * p->npair)) &&
-            (!starts32 || (alloc((void**)&p->d_lc32, sizeof(int) * nchain) &&
-                           alloc((void**)&p->d_start32, sizeof(float4) * nchain))) &&
             alloc(&p->d_spec, cs * (size_t)nbatch * p->nspec) &&
             alloc(&p->d_F, cs * (size_t)nbatch * p->nring * (mmax + 1)) &&
             alloc((void**)&p->d_status, sizeof(int));
   if (!ok) {
     plan_free(p);
     return HPX_ERR_NOMEM;
+  }
+  if (starts32) {  // behind the others: two allocations fewer
+    p->d_lc32 = p->d_lc + nchain;
+    p->d_start32 = p->d_start + nchain;
   }
   cudaStream_t s;
   cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);

@@ -238,11 +238,13 @@ static cudaError_t run_analysis(hpx_plan_s* p, const void* map, void* alm, bool 
     return launch_r2c<T>(p, static_cast<const T*>(map), s);
   });
   if (e != cudaSuccess) return e;
-  hpx_plan_s view;
-  if (staged_view(p, s, &view)) {
-    e = run_tc_analysis(&view, alm, weighted, mfac, s);
-    p->stage_next = view.stage_next;
-    return e;
+  if (p->gen_wide) {
+    hpx_plan_s view;
+    if (staged_view(p, s, &view)) {
+      e = run_tc_analysis(&view, alm, weighted, mfac, s);
+      p->stage_next = view.stage_next;
+      return e;
+    }
   }
   if (p->tc_nn_a) return run_tc_analysis(p, alm, weighted, mfac, s);
   if (gen_analysis(p)) {
